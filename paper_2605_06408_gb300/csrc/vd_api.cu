@@ -20,7 +20,6 @@ namespace {
 
 constexpr int kStride = 64;      // neighbour row stride of the register-resident pass
 constexpr int kAmbCap = 1 << 16; // cells recorded with an FP64-ambiguous sign test
-constexpr int kHistEntries = 256 * 2 * kSortBlocksMax;
 
 size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
@@ -175,7 +174,7 @@ static Layout make_layout(int64_t n, int num_sms) {
   L.add(sizeof(int) * n);              // 3 vals_a
   L.add(sizeof(int) * n);              // 4 vals_b
   L.add(sizeof(int) * n);              // 5 inv_perm
-  L.add(sizeof(unsigned) * kHistEntries);  // 6 hist
+  L.add(sort_scratch_bytes(n));        // 6 sort scratch
   L.add(sizeof(int) * n);              // 7 left
   L.add(sizeof(int) * n);              // 8 right
   L.add(sizeof(int) * 2 * n);          // 9 parent
@@ -365,9 +364,10 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   // 1. keys: (set, weight stratum, Morton code in the set's box); input validation
   e = launch_weight_range(w, n, ctx->sets_dev, nsets, ctx->wrange, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
+  if (launch_sort_clear(ctx->hist, n, s) != cudaSuccess) return VD_ERR_CUDA;
   const int bin_shift = nsets > 1 ? 51 : 60;
   e = launch_pack_keys(xyz, w, n, ctx->sets_dev, nsets, set_shift, bin_shift, ctx->wrange, ctx->keys_a,
-                       ctx->vals_a, ctx->st, s);
+                       ctx->vals_a, ctx->hist, ctx->st, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
   mark(ctx, 1, s);
   // 2. radix sort of (key, index)
@@ -376,7 +376,7 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   int* v0 = ctx->vals_a;
   int* v1 = ctx->vals_b;
   int bits = nsets > 1 ? 64 : 63;
-  e = radix_sort_pairs(k0, k1, v0, v1, ctx->hist, n, bits, s);
+  e = radix_sort_pairs(k0, k1, v0, v1, ctx->hist, n, bits, ctx->st, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
   ctx->keys_sorted = k0;
   ctx->perm = v0;
@@ -440,7 +440,7 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   ctx->ev_valid = ctx->cfg.timing != 0;
   ctx->ev_backward = false;
   int passes = (bits + 7) / 8;
-  ctx->launches = (w ? 1 : 0) + 1 + 3 * passes + 3 + (n >= 2 ? 4 : 1) + 2 + 3 +
+  ctx->launches = (w ? 1 : 0) + 1 + passes + 3 + (n >= 2 ? 4 : 1) + 2 + 3 +
                   (out->neighbors && out->nnz_capacity > 0) + 1 + (knn ? 1 : 0);
   return VD_OK;
 }

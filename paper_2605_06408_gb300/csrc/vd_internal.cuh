@@ -240,7 +240,7 @@ struct BvhBuffers {
   uint64_t* keys_alt;
   int* vals;
   int* vals_alt;
-  unsigned* hist;      // [256 * 2 * kSortBlocksMax]
+  unsigned* hist;      // the sort's scratch (sort_scratch_bytes)
   // Karras tree
   int* left;
   int* right;
@@ -298,8 +298,7 @@ struct CellBuffers {
   const int* knn;        // [n * kKnn] nearest sites (sorted indices, -1 = none) for warm_start = 2
 };
 
-constexpr int kSortThreads = 512;
-constexpr int kSortBlocksMax = 1024;
+constexpr int kSortHist = 8 * 256 + 64;  // digit counts and tickets at the head of the sort's scratch
 
 struct BackBuffers {
   CellBuffers c;
@@ -326,10 +325,12 @@ struct BackBuffers {
 cudaError_t launch_weight_range(const float* w, int n, const SetInfo* sets, int nsets, unsigned* wr,
                                 cudaStream_t s);
 cudaError_t launch_pack_keys(const float* xyz, const float* w, int n, const SetInfo* sets, int nsets, int set_shift,
-                             int bin_shift, const unsigned* wr, uint64_t* keys, int* vals, DevStatus* st,
+                             int bin_shift, const unsigned* wr, uint64_t* keys, int* vals, unsigned* hist, DevStatus* st,
                              cudaStream_t s);
-cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, int*& vals_alt, unsigned* hist,
-                             int n, int bits, cudaStream_t s);
+size_t sort_scratch_bytes(int64_t n);
+cudaError_t launch_sort_clear(unsigned* scratch, int n, cudaStream_t s);
+cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, int*& vals_alt, unsigned* scratch, int n,
+                             int bits, DevStatus* st, cudaStream_t s);
 cudaError_t launch_gather_sites(const float* xyz, const float* w, const int* perm, int n, const SetInfo* sets,
                                 const uint64_t* keys, int set_shift, int nsets, float4* sites, cudaStream_t s);
 cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, int leaf_size, BvhBuffers& b,
