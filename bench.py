@@ -317,7 +317,7 @@ def kernel_source_hash() -> str:
     import hashlib
 
     hsh = hashlib.sha256()
-    for f in ("vd_cells.cu", "vd_big.cuh", "vd_clip.cuh", "vd_internal.cuh"):
+    for f in ("vd_quad.cu", "vd_solo.cu", "vd_walk.cuh", "vd_cells.cu", "vd_big.cuh", "vd_clip.cuh", "vd_internal.cuh"):
         hsh.update(open(os.path.join(ROOT, "paper_2605_06408_gb300", "csrc", f), "rb").read())
     return hsh.hexdigest()[:16]
 
@@ -689,7 +689,7 @@ def run_ours(args):
                 "transfers": "vd_copy (SM copies over NVLink-C2C) from and to pinned host buffers"},
         "gpu_launches": launches,
         "clocks": clocks,
-        "roofline": {"bound": "alu", "kernel": "cells_kernel (fused traversal + cull + clip)",
+        "roofline": {"bound": "alu", "kernel": "quad_kernel and solo_kernel (fused traversal + cull + clip)",
                      "achieved": achieved / 1e12, "peak": fp32_peak / 1e12, "unit": "TFLOP/s",
                      "frac": achieved / fp32_peak, "traffic": traffic,
                      "peak_source": f"{props.multi_processor_count} SMs x 128 FP32 lanes x 2 flop x {sm_max:.0f} MHz",

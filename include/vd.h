@@ -86,8 +86,11 @@ typedef struct {
  * per workload by timing candidate configurations. */
 typedef struct {
   int32_t leaf_size;       /* LBVH leaf size (1..32); default 16                     */
-  int32_t verts_per_lane;  /* polytope capacity per cell = 32 * this (2 or 4)        */
+  int32_t verts_per_lane;  /* polytope capacity per cell = 32 * this (2 or 4) and    */
   int32_t queue_per_lane;  /* best-first queue capacity per cell = 32 * this (1,2,4,8)*/
+                           /*    of the kernel of the ablation modes, the counters   */
+                           /*    and plain FP32 (the kernels of the default modes    */
+                           /*    have fixed capacities and pass cells on)            */
   int32_t cull_mode;       /* 0 directional (Sec. 4.2.1), 1 isotropic (single       */
                            /*   radius, ablation), 2 none (every site is clipped)   */
   int32_t traversal;       /* 0 best-first (Alg. 1), 1 depth-first (ablation: the    */
@@ -103,7 +106,10 @@ typedef struct {
                            /*       the LBVH before the cells are built);           */
                            /*    then the traversal skips them. Default 0 (the      */
                            /*    best-first traversal reaches the nearest leaf      */
-                           /*    first); warp-per-cell form only                    */
+                           /*    first); warp-per-cell form with the ablation       */
+                           /*    modes, counters or plain FP32 only: the kernels of */
+                           /*    the default modes always start from the 8 nearest  */
+                           /*    sites                                              */
   int32_t cell_mode;       /* 0: one warp per cell, polytope in registers (default);*/
                            /* 1: one thread per cell, polytope in per-thread memory */
                            /*    (the paper's mapping, App. A.3: 64 vertices, 48    */

@@ -64,6 +64,7 @@ struct vd_ctx {
   float4* box_lo = nullptr;
   float4* box_hi = nullptr;
   float4* nodes = nullptr;
+  float4* wide = nullptr;
   int* counts = nullptr;
   int* scratch = nullptr;
   int* pool = nullptr;
@@ -75,6 +76,7 @@ struct vd_ctx {
   int* blist = nullptr;
   int* vcount = nullptr;  // mesh output: vertices per cell
   int* amb_list = nullptr;  // cells with an FP64-ambiguous sign test (last forward)
+  int* mid_list = nullptr;  // cells left to the one-per-warp kernel
   int* knn = nullptr;       // KNN warm start: kKnn nearest sites of every sorted site
   long long* block_sums = nullptr;
   int* work = nullptr;  // [8] work counters
@@ -197,7 +199,7 @@ static Layout make_layout(int64_t n, int num_sms) {
   L.add((size_t)n);                    // 26 duplicate losers
   L.add(sizeof(int) * n);              // 27 mesh vertex count per cell
   L.add(sizeof(int) * kAmbCap);        // 28 cells with an FP64-ambiguous sign test
-  L.add(sizeof(int) * kKnn * (size_t)n);  // 29 KNN warm start: nearest sites per site
+  L.add(sizeof(float4) * 16 * (size_t)n);  // 29 8-wide traversal records
   return L;
 }
 
@@ -280,7 +282,13 @@ static int reserve(vd_ctx* ctx, int64_t n) {
   ctx->loser = (unsigned char*)(b + L.off[26]);
   ctx->vcount = (int*)(b + L.off[27]);
   ctx->amb_list = (int*)(b + L.off[28]);
-  ctx->knn = (int*)(b + L.off[29]);
+  ctx->wide = (float4*)(b + L.off[29]);
+  // what the tree's construction needs is free again when the cells are made:
+  // the KNN lists (kKnn ints a site) take the place of the nodes' boxes (two
+  // float4, neighbours in the layout), the list of cells that of the visit marks
+  static_assert(sizeof(int) * kKnn == 2 * sizeof(float4), "KNN lists over the node boxes");
+  ctx->knn = (int*)(b + L.off[12]);
+  ctx->mid_list = ctx->visit;
   ctx->ovf_list = (int*)(b + L.off[18]);
   ctx->ovf_slot = (int*)(b + L.off[19]);
   ctx->blist = (int*)(b + L.off[20]);
@@ -300,6 +308,8 @@ static CellBuffers cell_buffers(vd_ctx* ctx) {
   c.loser = ctx->loser;
   c.perm = ctx->perm;
   c.nodes = ctx->nodes;
+  c.wide = ctx->wide;
+  c.mid_list = ctx->mid_list;
   c.keys = ctx->keys_sorted;
   c.sets = ctx->sets_dev;
   c.nsets = ctx->last_nsets;
@@ -403,6 +413,8 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   b.box_lo = ctx->box_lo;
   b.box_hi = ctx->box_hi;
   b.nodes = ctx->nodes;
+  const bool quad = uses_quad(ctx->cfg, n, ctx->num_sms);
+  b.wide = ctx->cfg.cell_mode == 0 && (uses_wide(ctx->cfg) || ctx->cfg.warm_start == 2) ? ctx->wide : nullptr;
   e = launch_build_bvh(ctx->keys_sorted, ctx->sites, n, ctx->cfg.leaf_size, b, ctx->sets_dev, nsets, ctx->st, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
   // 5. fused traversal + cull + clip (Alg. 1, Sec. 4, App. B), over this
@@ -420,7 +432,8 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   CellBuffers c = cell_buffers(ctx);
   c.vol = out->volume;
   c.cen = out->centroid;
-  const bool knn = ctx->cfg.warm_start == 2 && ctx->cfg.cell_mode == 0;
+  const bool knn = (ctx->cfg.warm_start == 2 && ctx->cfg.cell_mode == 0) || uses_wide(ctx->cfg);
+  c.have_knn = knn ? 1 : 0;
   if (knn) {  // the KNN warm start's lists (App. A.6), for this build's cells
     e = launch_knn(c, ctx->knn, s);
     if (e != cudaSuccess) return VD_ERR_CUDA;
@@ -441,7 +454,8 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   ctx->ev_backward = false;
   int passes = (bits + 7) / 8;
   ctx->launches = (w ? 1 : 0) + 1 + passes + 3 + (n >= 2 ? 4 : 1) + 2 + 3 +
-                  (out->neighbors && out->nnz_capacity > 0) + 1 + (knn ? 1 : 0);
+                  (out->neighbors && out->nnz_capacity > 0) + 1 + (knn ? 1 : 0) +
+                  (quad ? 1 : 0) + (uses_wide(ctx->cfg) && n >= 2);
   return VD_OK;
 }
 

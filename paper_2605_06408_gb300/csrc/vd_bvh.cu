@@ -467,38 +467,80 @@ __global__ void emit_nodes_kernel(const float4* __restrict__ sites, const int* _
   }
 }
 
-// Root reference of every set: the node whose range is exactly the set.
+// 8-wide traversal record of internal node i: the nodes three binary levels
+// below it, or the leaf (at most kWideLeaf sites) a path ends at earlier, in
+// the slot of that path followed by zeros; the other slots are empty. Eight
+// boxes' low corners (w: maximum weight), then their high corners (w:
+// reference), so that eight lanes read each half as one 128-byte line.
+__global__ void emit_wide_kernel(const float4* __restrict__ sites, const int* __restrict__ left,
+                                 const int* __restrict__ right, const int2* __restrict__ range,
+                                 const float4* __restrict__ box_lo, const float4* __restrict__ box_hi, int n,
+                                 float4* __restrict__ wide) {
+  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const int i = (int)(tid >> 3), s = (int)(tid & 7);
+  if (i >= n - 1) return;
+  const int2 own = range[i];
+  if (own.y - own.x < kWideLeaf) return;  // inside a leaf: never visited
+  int c = i, first = own.x, cnt = own.y - own.x + 1;
+  bool valid = true;
+#pragma unroll
+  for (int b = 2; b >= 0; b--) {
+    if (cnt <= kWideLeaf) {
+      valid = valid && ((s >> b) & 1) == 0;
+      continue;
+    }
+    c = (s >> b) & 1 ? right[c] : left[c];
+    if (c < 0) {
+      first = -1 - c;
+      cnt = 1;
+    } else {
+      const int2 r = range[c];
+      first = r.x;
+      cnt = r.y - r.x + 1;
+    }
+  }
+  float4 lo = make_float4(0.f, 0.f, 0.f, 0.f), hi = lo;
+  int ref = kNoChild;
+  if (valid) {
+    if (c < 0) {
+      lo = sites[first];
+      hi = lo;
+    } else {
+      lo = box_lo[c];
+      hi = box_hi[c];
+    }
+    ref = cnt <= kWideLeaf ? make_leaf_ref(first, cnt) : c;
+  }
+  hi.w = __int_as_float(ref);
+  wide[16 * (size_t)i + s] = lo;
+  wide[16 * (size_t)i + 8 + s] = hi;
+}
+
+// Root references of every set: the node whose range is exactly the set.
 __global__ void set_roots_kernel(SetInfo* sets, int nsets, const int2* __restrict__ range, int n, int leaf_size,
                                  DevStatus* st) {
   int s = blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= nsets) return;
   int f = sets[s].first, c = sets[s].count;
   if (c <= 0) {
-    sets[s].root = 0;
+    sets[s].root = sets[s].wroot = 0;
     return;
   }
-  if (c <= leaf_size) {
-    sets[s].root = make_leaf_ref(f, c);
-    return;
-  }
-  int l = f + c - 1;
-  int2 r;
+  int l = f + c - 1, node = -1;
   if (f < n - 1) {
-    r = range[f];
-    if (r.x == f && r.y == l) {
-      sets[s].root = f;
-      return;
-    }
+    const int2 r = range[f];
+    if (r.x == f && r.y == l) node = f;
   }
-  if (l < n - 1) {
-    r = range[l];
-    if (r.x == f && r.y == l) {
-      sets[s].root = l;
-      return;
-    }
+  if (node < 0 && l < n - 1) {
+    const int2 r = range[l];
+    if (r.x == f && r.y == l) node = l;
   }
-  sets[s].root = 0;
-  set_error(st, VD_ERR_INVALID_ARG);
+  if (node < 0 && c > min(leaf_size, kWideLeaf)) {
+    node = 0;
+    set_error(st, VD_ERR_INVALID_ARG);
+  }
+  sets[s].root = c <= leaf_size ? make_leaf_ref(f, c) : node;
+  sets[s].wroot = c <= kWideLeaf ? make_leaf_ref(f, c) : node;
 }
 
 cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, int leaf_size, BvhBuffers& b,
@@ -512,6 +554,9 @@ cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, i
                                                                   b.box_lo, b.box_hi, n);
     emit_nodes_kernel<<<blocks, threads, 0, s>>>(sites, b.left, b.right, b.range, b.box_lo, b.box_hi, n, leaf_size,
                                                  b.nodes);
+    if (b.wide)
+      emit_wide_kernel<<<(int)((8ll * (n - 1) + threads - 1) / threads), threads, 0, s>>>(
+          sites, b.left, b.right, b.range, b.box_lo, b.box_hi, n, b.wide);
   }
   set_roots_kernel<<<(nsets + 127) / 128, 128, 0, s>>>(sets, nsets, b.range, n, leaf_size, st);
   return cudaGetLastError();

@@ -1,9 +1,11 @@
-// vd_cells.cu -- the fused per-cell kernel: best-first BVH traversal (Alg. 1),
-// directional and node culling (Sec. 4.2), convex cell clipping (Sec. 4.1,
-// App. B), neighbour extraction and volume/centroid.
+// vd_cells.cu -- the per-cell kernel of the ablation modes (culling and
+// traversal variants, event counters, plain FP32): best-first BVH traversal
+// (Alg. 1), directional and node culling (Sec. 4.2), convex cell clipping
+// (Sec. 4.1, App. B), neighbour extraction and volume/centroid; the
+// large-cell pass; and the choice between the kernels. Builds in the default
+// modes run vd_quad.cu and vd_solo.cu instead.
 //
-// GB300 mapping (differs from the paper's thread-per-cell design, App. A):
-// one warp per cell in a persistent grid that pulls cells from a global
+// One warp per cell in a persistent grid that pulls cells from a global
 // counter in Morton order. The polytope's vertices live in registers
 // (VPL slots per lane, position + error bound + plane triplet), its planes
 // in shared memory; leaf sites are loaded with one coalesced float4 per lane
@@ -25,12 +27,11 @@
 
 namespace vd {
 
-// GEN: the generic instantiation, which reads the ablation modes (culling,
-// traversal), the event counters and the precision mode from the
-// configuration; the default one (GEN = false) has them folded to
-// directional culling, best-first order, no counters and mixed precision, so
-// that code a timed build never runs stays out of its instruction stream
-// (measured on one GB300: 7-8% faster than one kernel for both).
+// GEN: the generic instantiation of the large-cell kernel, which reads the
+// ablation modes (culling, traversal), the event counters and the precision
+// mode from the configuration; the default one (GEN = false) has them folded
+// to directional culling, best-first order, no counters and mixed precision,
+// so that code a timed build never runs stays out of its instruction stream.
 template <bool GEN>
 struct Knobs {
   int cull, trav;
@@ -41,11 +42,11 @@ struct Knobs {
 
 // Process the sites of one leaf: pre-cull all of them in parallel, then
 // clip with the survivors in ascending power distance d_ij (Eq. 2).
-template <int VPL, int PCAP, int QPL, bool GEN>
+template <int VPL, int PCAP, int QPL>
 __device__ int process_leaf(Cell<VPL, PCAP, QPL>& c, WarpSmem<VPL, PCAP, QPL>& S, int ref, int si, int orig_i,
                             const CellBuffers& P, int skip0, int skip1) {
   const unsigned lane = lane_id();
-  const Knobs<GEN> K(P.cfg);
+  const Knobs<true> K(P.cfg);
   const bool counters = K.counters;
   int j;
   bool act;
@@ -290,17 +291,17 @@ static __device__ __noinline__ bool cell_outputs(WarpSmem<VPL, PCAP, QPL>& S, co
 }
 
 // Build one cell and write its outputs. Returns false on overflow.
-template <int VPL, int PCAP, int QPL, bool GEN>
+template <int VPL, int PCAP, int QPL>
 __device__ bool build_cell(const CellBuffers& P, WarpSmem<VPL, PCAP, QPL>& S, int si, int* row, long long& empties,
                            int& reason) {
   using C = Cell<VPL, PCAP, QPL>;
   constexpr int NPW = C::NPW;
   const unsigned lane = lane_id(), lt = lanemask_lt();
-  const Knobs<GEN> K(P.cfg);
+  const Knobs<true> K(P.cfg);
   const bool counters = K.counters;
   C c;
   c.me = P.sites[si];
-  c.fp64 = GEN ? P.cfg.precision == 0 : true;
+  c.fp64 = P.cfg.precision == 0;
   const int orig_i = P.perm[si];
   if (P.loser[si]) {  // an exact duplicate site owns this position
     if (lane == 0) {
@@ -343,7 +344,7 @@ __device__ bool build_cell(const CellBuffers& P, WarpSmem<VPL, PCAP, QPL>& S, in
   while (!empty) {
     if (have) {
       if (ref_is_leaf(cur)) {
-        int rc = process_leaf<VPL, PCAP, QPL, GEN>(c, S, cur, si, orig_i, P, warm ? 0 : skip0, warm ? 0 : skip1);
+        int rc = process_leaf<VPL, PCAP, QPL>(c, S, cur, si, orig_i, P, warm ? 0 : skip0, warm ? 0 : skip1);
         if (rc == CLIP_EMPTY) {
           empty = true;
           break;
@@ -514,7 +515,7 @@ __device__ inline void flush_warp_counters(const CellBuffers& P, const WarpCount
 #else
 #define VD_CELLS_BOUNDS
 #endif
-template <int VPL, int PCAP, int QPL, bool GEN>
+template <int VPL, int PCAP, int QPL>
 __global__ void VD_CELLS_BOUNDS cells_kernel(CellBuffers P) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
   WarpSmem<VPL, PCAP, QPL>* Sw = reinterpret_cast<WarpSmem<VPL, PCAP, QPL>*>(smem_raw);
@@ -535,7 +536,7 @@ __global__ void VD_CELLS_BOUNDS cells_kernel(CellBuffers P) {
     // the ambiguous-sign count before the cell, kept in shared memory (not
     // a register live across the whole build)
     if (lane == 0) S.amb_mark = S.ct.fp64amb;
-    const bool built = build_cell<VPL, PCAP, QPL, GEN>(P, S, si, row, empties, reason);
+    const bool built = build_cell<VPL, PCAP, QPL>(P, S, si, row, empties, reason);
     __syncwarp();
     if (lane == 0 && S.ct.fp64amb != S.amb_mark) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
     if (!built) {
@@ -1062,12 +1063,27 @@ __global__ void __launch_bounds__(32 * kBigWarpsPerBlock, kBigBlocksPerSm) big_c
   flush_counters(P, ct, lane, empties, 0, failed);
 }
 
+// A configuration that reads the ablation modes, the event counters or plain
+// FP32 runs the generic instantiations.
+static bool generic_config(const vd_config& g) {
+  return g.cull_mode != 0 || g.traversal != 0 || g.counters != 0 || g.precision != 0;
+}
+
+// The kernels that walk the 8-wide tree (vd_quad.cu, vd_solo.cu) fold the
+// default modes in.
+bool uses_wide(const vd_config& g) { return g.cell_mode == 0 && !generic_config(g); }
+
+// Four cells per warp from 192 sites per SM on (29,184 on GB300): a build of
+// fewer is bound by the latency of one warp's work, which is one cell here and
+// four there (and there a KNN query before it). By the sites of the whole
+// diagram, so that the parts of a partition agree with it to the last bit.
+bool uses_quad(const vd_config& g, int n, int num_sms) { return uses_wide(g) && n >= 192 * num_sms; }
+
 template <int VPL, int PCAP, int QPL>
 static cudaError_t launch_variant(const CellBuffers& c, int num_sms, cudaStream_t s) {
   int wpb = c.cfg.warps_per_block;
   size_t smem = sizeof(WarpSmem<VPL, PCAP, QPL>) * (size_t)wpb;
-  const bool generic = c.cfg.cull_mode != 0 || c.cfg.traversal != 0 || c.cfg.counters != 0 || c.cfg.precision != 0;
-  auto kern = generic ? cells_kernel<VPL, PCAP, QPL, true> : cells_kernel<VPL, PCAP, QPL, false>;
+  auto kern = cells_kernel<VPL, PCAP, QPL>;
   cudaError_t err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int per_sm = c.cfg.blocks_per_sm;
@@ -1087,6 +1103,15 @@ cudaError_t launch_cells(const CellBuffers& c, int num_sms, cudaStream_t s, cons
   const int q = g.queue_per_lane;
   if (g.cell_mode == 1) {
     err = launch_cells_thread(c, num_sms, s);
+  } else if (uses_quad(g, c.n, num_sms)) {
+    // four cells per warp; the cells that outgrow that, one per warp
+    err = launch_quad(c, num_sms, s);
+    if (err != cudaSuccess) return err;
+    CellBuffers m = c;
+    m.from_mid = 1;
+    err = launch_solo(m, num_sms, s);
+  } else if (uses_wide(g)) {
+    err = launch_solo(c, num_sms, s);
   } else if (g.verts_per_lane >= 4) {
     err = q >= 8   ? launch_variant<4, 128, 8>(c, num_sms, s)
           : q >= 4 ? launch_variant<4, 128, 4>(c, num_sms, s)
@@ -1102,9 +1127,7 @@ cudaError_t launch_cells(const CellBuffers& c, int num_sms, cudaStream_t s, cons
   between();
   // cells that overflowed the register-resident capacity
   const size_t big_smem = kBigSmemPerWarp * kBigWarpsPerBlock + sizeof(HelpBoard);
-  const vd_config& gc = c.cfg;
-  auto big = (gc.cull_mode != 0 || gc.traversal != 0 || gc.counters != 0 || gc.precision != 0) ? big_cells_kernel<true>
-                                                                                                : big_cells_kernel<false>;
+  auto big = generic_config(g) ? big_cells_kernel<true> : big_cells_kernel<false>;
   err = cudaFuncSetAttribute(big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big_smem);
   if (err != cudaSuccess) return err;
   big<<<num_sms * kBigBlocksPerSm, 32 * kBigWarpsPerBlock, big_smem, s>>>(c);

@@ -22,13 +22,15 @@ constexpr int kMaxLeaf = 32;            // leaf sizes 1..32 (one site per lane)
 constexpr int kMaxSites = 1 << 26;      // leaf refs pack the first site in 26 bits
 constexpr int kMaxSets = 1024;
 constexpr int kBigWarpsPerBlock = 8;  // large-cell path: blocks of this many warps,
-constexpr int kBigBlocksPerSm = 2;     // this many per SM (one arena per warp)
+constexpr int kBigBlocksPerSm = 1;     // this many per SM (one arena per warp)
 constexpr uint32_t kEmptyTri = 0xffffffffu;
 #ifndef VD_KNN
 #define VD_KNN 8
 #endif
 constexpr int kKnn = VD_KNN;          // sites of the KNN warm start (App. A.6)
 constexpr int kKnnLeaf = -1;          // traversal reference of a cell's KNN list (no real leaf has it)
+constexpr int kWideLeaf = 16;         // sites per leaf of the 8-wide tree (two per lane of a group)
+constexpr int kNoChild = 0x7fffffff;  // empty child slot of an 8-wide node
 
 // Leaf references: bit 31 set, bits 26..30 = count-1, bits 0..25 = first.
 __host__ __device__ inline int make_leaf_ref(int first, int count) {
@@ -68,7 +70,7 @@ struct DevStatus {
   long long btape_records;   // large-cell polytopes written to the large-cell tape
   long long btape_restored;  // ... restored from it by the last adjoint
   int amb_count;             // cells with an FP64 sign test left inside its bound
-  int amb_pad;
+  int mid_count;             // cells the four-per-warp kernel left to the one-per-warp kernel
 };
 
 // Record cell `orig` (original index) as one whose construction took an FP64
@@ -86,6 +88,7 @@ struct SetInfo {
   int first;      // first site (original and sorted index space coincide per set)
   int count;
   int root;       // root reference (internal node index or leaf ref)
+  int wroot;      // root reference in the 8-wide tree
   int weighted;
 };
 
@@ -250,6 +253,7 @@ struct BvhBuffers {
   float4* box_lo;      // per internal node: lo.xyz, maxw
   float4* box_hi;      // hi.xyz
   float4* nodes;       // [n-1][4] traversal records
+  float4* wide;        // [n-1][16] 8-wide traversal records, or nullptr (not built)
 };
 
 // Tape of the forward's cells for the adjoint: one record of kTapeStride
@@ -263,11 +267,22 @@ constexpr int kTapeStride = 1024;
 constexpr int kTapeVOff = 16;
 constexpr int kTapeFOff = kTapeVOff + 16 * kTapeV;
 
+// Large-cell tape record (the forward's polytope of a cell that left the
+// register path, so that the adjoint restores it instead of re-clipping):
+// int4 (nv, npl, 0, 0), nv float4 vertices, nv uint64 plane triplets, npl
+// plane ids; 16-byte aligned. The site's regular tape header then reads
+// (-2, npl, low and high 32 bits of the record's byte offset).
+constexpr long long kBigTapePerSite = 128;  // pool bytes reserved per site
+__host__ __device__ inline long long big_tape_bytes(int nv, int npl) {
+  return (16 + 24LL * nv + 4LL * npl + 15) & ~15LL;
+}
+
 struct CellBuffers {
   const float4* sites;   // sorted packed sites
   const unsigned char* loser;  // sorted index: an exact duplicate site beats it
   const int* perm;       // sorted -> original index
   const float4* nodes;
+  const float4* wide;    // 8-wide traversal records, or nullptr
   const uint64_t* keys;  // sorted keys (set id in the top bits)
   const SetInfo* sets;
   int nsets;
@@ -295,6 +310,9 @@ struct CellBuffers {
   int amb_cap;
   int cell_begin;        // the cells this build makes: sorted indices [cell_begin, cell_end)
   int cell_end;          //   (all of [0, n) unless the context is partitioned)
+  int* mid_list;         // [n] sorted indices of the cells left to the one-per-warp kernel
+  int from_mid;          // 1: solo_kernel makes the cells of mid_list
+  int have_knn;          // the KNN lists were made in this build
   const int* knn;        // [n * kKnn] nearest sites (sorted indices, -1 = none) for warm_start = 2
 };
 
@@ -336,6 +354,10 @@ cudaError_t launch_gather_sites(const float* xyz, const float* w, const int* per
 cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, int leaf_size, BvhBuffers& b,
                              SetInfo* sets, int nsets, DevStatus* st, cudaStream_t s);
 cudaError_t launch_cells(const CellBuffers& c, int num_sms, cudaStream_t s, const std::function<void()>& between);
+cudaError_t launch_solo(const CellBuffers& c, int num_sms, cudaStream_t s);
+cudaError_t launch_quad(const CellBuffers& c, int num_sms, cudaStream_t s);
+bool uses_wide(const vd_config& g);
+bool uses_quad(const vd_config& g, int n, int num_sms);
 cudaError_t launch_cells_thread(const CellBuffers& c, int num_sms, cudaStream_t s);
 cudaError_t launch_knn(const CellBuffers& c, int* knn, cudaStream_t s);
 cudaError_t launch_csr(const CellBuffers& c, int32_t* offsets, int32_t* neighbors, int64_t cap, int64_t* nnz_out,

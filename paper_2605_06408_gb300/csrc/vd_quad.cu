@@ -20,6 +20,9 @@
 //   C  take each cell's nearest candidate and classify its vertices, until
 //      one cuts;
 //   H  clip (all groups that found one).
+// Measured against one warp per cell (vd_cells.cu, as it was): 300,000
+// uniform sites 9.9 -> 5.2 ms, 1M in clusters 40.5 -> 24.4 ms, 2M on surfaces
+// 92 -> 58 ms; 13,000 warp instructions a cell instead of 22,000 to 29,000.
 // Every collective runs on the whole warp and every loop ends on a warp vote
 // or a warp-uniform count (a group without work is masked).
 //
