@@ -330,6 +330,9 @@ struct BackBuffers {
   int list_cap;
   int* work;            // [2]
   const char* tape;     // the forward's tape, or nullptr (re-clip every cell)
+  int* list2;           // cells that the tape does not hold
+  int* list2_count;
+  int* list2_next;      // work counter over them
   // mesh output and vertex gradients
   int mode;              // 0: gradients; 1: vertex count per cell; 2: vertex output
   int* vcount;           // [n] by original index (mode 1)
@@ -355,6 +358,7 @@ cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, i
                              SetInfo* sets, int nsets, DevStatus* st, cudaStream_t s);
 cudaError_t launch_cells(const CellBuffers& c, int num_sms, cudaStream_t s, const std::function<void()>& between);
 cudaError_t launch_solo(const CellBuffers& c, int num_sms, cudaStream_t s);
+cudaError_t launch_solo_brute(const CellBuffers& c, int num_sms, cudaStream_t s);
 cudaError_t launch_quad(const CellBuffers& c, int num_sms, cudaStream_t s);
 bool uses_wide(const vd_config& g);
 bool uses_quad(const vd_config& g, int n, int num_sms);

@@ -21,6 +21,7 @@ namespace vd {
 namespace {
 
 constexpr int kSV = 192;  // vertices (their slot takes a byte of otri)
+constexpr int kSBrute = 128;  // vertices without a tree (larger cells are not made there)
 constexpr int kSP = 128;  // planes (a byte of a triplet)
 constexpr int kSQ = 96;   // queue entries (7 bits of the key)
 constexpr int kSC = 96;   // candidates
@@ -298,6 +299,10 @@ __device__ __forceinline__ int solo_pop(SoloCell& S, int& qn, uint32_t& todo) {
   return ref;
 }
 
+// BRUTE: no tree; every site of one set is read, 64 a step, after the nearest
+// of every 32nd (one per lane) have clipped the cell (vd_cells_noalloc). A
+// cell that does not fit is marked there and then.
+template <bool BRUTE>
 __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
   extern __shared__ __align__(16) unsigned char solo_smem[];
   SoloCell& S = reinterpret_cast<SoloCell*>(solo_smem)[threadIdx.x >> 5];
@@ -307,6 +312,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
   unsigned ct64 = 0, ctamb = 0, ctrefv = 0, ctrefvol = 0, ctempty = 0, ctovf = 0;
   int* const work = P.from_mid ? &P.work[5] : &P.work[0];
   const int total = P.from_mid ? P.st->mid_count : P.cell_end - P.cell_begin;
+  auto original = [&](int j) { return BRUTE ? j : P.perm[j]; };
 
   while (true) {
     int item = 0;
@@ -315,7 +321,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
     if (item >= total) break;
     const int si = P.from_mid ? P.mid_list[item] : P.cell_begin + item;
     const float4 me = P.sites[si];
-    const int orig = P.perm[si];
+    const int orig = original(si);
     const SetInfo& SI = P.sets[P.nsets > 1 ? (int)(P.keys[si] >> P.set_shift) : 0];
     const float* box = SI.lo;
     const bool weighted = SI.weighted != 0;
@@ -353,7 +359,18 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
     // site's 32 neighbours in the sorted order (one coalesced load)
     const bool knn = P.have_knn != 0;
     int kid = -1, w0 = 0, w1 = 0;
-    if (knn) {
+    if (BRUTE) {
+      float best = INFINITY;
+      for (int j = lane; j < P.n; j += 32) {
+        const float4 q = P.sites[j];
+        const float dx = q.x - me.x, dy = q.y - me.y, dz = q.z - me.z;
+        const float d = fmaf(dx, dx, fmaf(dy, dy, dz * dz)) - q.w;
+        if (d < best && j != si) {
+          best = d;
+          kid = j;
+        }
+      }
+    } else if (knn) {
       if (lane < kKnn) kid = P.knn[(size_t)si * kKnn + lane];
     } else {
       const int lo = SI.first, hi = SI.first + SI.count;
@@ -361,7 +378,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
       w1 = min(hi, w0 + 32);
     }
     {
-      const int j = knn ? kid : (w0 + lane < w1 && w0 + lane != si ? w0 + lane : -1);
+      const int j = BRUTE || knn ? kid : (w0 + lane < w1 && w0 + lane != si ? w0 + lane : -1);
       const uint32_t m = __ballot_sync(FULL, j >= 0);
       if (j >= 0) {
         const int at = __popc(m & lt);
@@ -375,7 +392,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
     uint32_t pend = 0;  // lanes whose child of the nodes visited last is a leaf still to be read
     int cref = 0;
     bool first = true, finished = false, dirty = true;
-    int steps = 0;  // node visits of the walk
+    int steps = 0;  // node visits of the walk (BRUTE: sites read)
     WalkBounds B;
 
 #pragma unroll 1
@@ -427,6 +444,22 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
       // ---- T: walk until the list is long or nothing is left
 #pragma unroll 1
       while (!first && cn <= kST) {
+        float4 q[2];
+        int j[2];
+        bool act[2], keep[2];
+        if constexpr (BRUTE) {
+          if (steps >= P.n) {
+            finished = true;
+            break;
+          }
+#pragma unroll
+          for (int r = 0; r < 2; r++) {
+            j[r] = steps + 32 * r + lane;
+            act[r] = (j[r] < P.n) & (j[r] != si);
+            q[r] = P.sites[act[r] ? j[r] : si];
+          }
+          steps += 64;
+        } else {
         if (pend == 0) {
           if (qn == 0 && cur < 0) {
             finished = true;
@@ -490,9 +523,6 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           continue;
         }
         // read up to four leaves, two at a time
-        float4 q[2];
-        int j[2];
-        bool act[2], keep[2];
 #pragma unroll
         for (int r = 0; r < 2; r++) {
           const int c0 = __ffs(pend) - 1;
@@ -504,6 +534,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           j[r] = leaf_first(ref) + (lane & 15);
           act[r] = (c >= 0) & ((lane & 15) < leaf_count(ref)) & (j[r] != si) & ((j[r] < w0) | (j[r] >= w1));
           q[r] = P.sites[act[r] ? j[r] : si];
+        }
         }
         bool dup = false;
 #pragma unroll
@@ -521,7 +552,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           for (int r = 0; r < 2; r++)
             if (act[r] && q[r].x == me.x && q[r].y == me.y && q[r].z == me.z) {
               keep[r] = false;
-              lose = lose || q[r].w > me.w || (q[r].w == me.w && P.perm[j[r]] < orig);
+              lose = lose || q[r].w > me.w || (q[r].w == me.w && original(j[r]) < orig);
             }
           if (__any_sync(FULL, lose)) {
             mode = S_EMPTY;
@@ -555,7 +586,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           const float nx = q.x - me.x, ny = q.y - me.y, nz = q.z - me.z;
           if (P.loser[id]) left = false;
           if (first && nx == 0.f && ny == 0.f && nz == 0.f) {  // a duplicate position among the first sites
-            if (left && (q.w > me.w || (q.w == me.w && P.perm[id] < orig))) mode = S_EMPTY;
+            if (left && (q.w > me.w || (q.w == me.w && original(id) < orig))) mode = S_EMPTY;
             left = false;
           }
           if (left) H = site_plane<float>(me.x, me.y, me.z, me.w, q.x, q.y, q.z, q.w);
@@ -564,7 +595,8 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           mode = S_EMPTY;
           break;
         }
-        if (knn && !first) {
+        if (BRUTE && !first) left = left & (id != __shfl_sync(FULL, kid, id & 31));
+        if (!BRUTE && knn && !first) {
 #pragma unroll
           for (int k = 0; k < kKnn; k++) left = left & (id != __shfl_sync(FULL, kid, k));
         }
@@ -668,13 +700,13 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
               const uint32_t ab = e == 0 ? (a | (b << 8)) : (e == 1 ? (b | (c << 8)) : (c | (a << 8)));
               if (is) {
                 const int slot = at < k ? (int)(S.otri[at] >> 24) : nv + (at - k);
-                if (slot < kSV) S.vt[slot] = ab | ((uint32_t)h << 16);
+                if (slot < (BRUTE ? kSBrute : kSV)) S.vt[slot] = ab | ((uint32_t)h << 16);
                 at++;
               }
             }
             m += __popc(m0) + __popc(m1) + __popc(m2);
           }
-          if (nv - k + m > kSV) {
+          if (nv - k + m > (BRUTE ? kSBrute : kSV)) {
             mode = S_FULL;
             break;
           }
@@ -763,13 +795,14 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
         const int f = 32 * w + lane;
         const bool isn = ((alive[w] >> lane) & 1u) && S.pid[f] >= 0;
         const uint32_t mk = __ballot_sync(FULL, isn);
-        if (isn) list[nb + __popc(mk & lt)] = (uint32_t)(P.perm[S.pid[f]] - SI.first);
+        if (isn) list[nb + __popc(mk & lt)] = (uint32_t)(original(S.pid[f]) - SI.first);
         nb += __popc(mk);
       }
       __syncwarp();
       // a list longer than a row goes to the pool
       int* row = P.scratch + (size_t)orig * P.stride;
-      if (nb > P.stride) {
+      if (BRUTE && nb > P.stride) mode = S_ROW;
+      if (!BRUTE && nb > P.stride) {
         unsigned long long off = 0;
         if (lane == 0) off = atomicAdd((unsigned long long*)&P.st->pool_used, (unsigned long long)nb);
         off = __shfl_sync(FULL, off, 0);
@@ -812,7 +845,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           }
         }
         __syncwarp();
-        if (P.tape) solo_tape(S, P, si, nv, nf, alive[0], alive[1], alive[2], alive[3]);
+        if (!BRUTE && P.tape) solo_tape(S, P, si, nv, nf, alive[0], alive[1], alive[2], alive[3]);
         __syncwarp();
         // volume and first moment: tetrahedra (c, g_f, v, w) as in cell_outputs
         const float inv = 1.0f / (float)nv;
@@ -888,14 +921,23 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
       P.cen[3 * (size_t)orig + 1] = me.y;
       P.cen[3 * (size_t)orig + 2] = me.z;
     }
-    if (mode > S_EMPTY && lane == 0) {  // to the large-cell pass
+    if (BRUTE && mode > S_EMPTY && lane == 0) {
+      const float nan = __int_as_float(0x7fc00000);
+      P.counts[orig] = -1;
+      P.vol[orig] = nan;
+      P.cen[3 * (size_t)orig] = nan;
+      P.cen[3 * (size_t)orig + 1] = nan;
+      P.cen[3 * (size_t)orig + 2] = nan;
+      set_error(P.st, VD_ERR_CELL_OVERFLOW);
+    }
+    if (!BRUTE && mode > S_EMPTY && lane == 0) {  // to the large-cell pass
       const int reason = mode == S_FULL ? OVF_VERTICES : mode == S_FAR ? OVF_QUEUE : mode == S_PLANES ? OVF_PLANES : OVF_NEIGHBORS;
       ctovf++;
       atomicAdd((unsigned long long*)&P.st->ovf_reason[reason], 1ull);
       P.ovf_list[atomicAdd(&P.st->ovf_count, 1)] = si;
       if (P.tape) *reinterpret_cast<int4*>(P.tape + (size_t)si * kTapeStride) = make_int4(-1, 0, 0, 0);
     }
-    if (__any_sync(FULL, ctamb != amb0) && lane == 0) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+    if (!BRUTE && __any_sync(FULL, ctamb != amb0) && lane == 0) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
     __syncwarp();
   }
   ct64 = __reduce_add_sync(FULL, ct64);
@@ -916,16 +958,28 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
 cudaError_t launch_solo(const CellBuffers& c, int num_sms, cudaStream_t s) {
   const int wpb = c.cfg.warps_per_block > 4 ? 4 : c.cfg.warps_per_block;
   const size_t smem = sizeof(SoloCell) * (size_t)wpb;
-  cudaError_t err = cudaFuncSetAttribute(solo_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t err = cudaFuncSetAttribute(solo_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return err;
   int per_sm = c.cfg.blocks_per_sm;
   if (per_sm <= 0) {
-    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solo_kernel, 32 * wpb, smem);
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, solo_kernel<false>, 32 * wpb, smem);
     if (err != cudaSuccess) return err;
     if (per_sm <= 0) per_sm = 1;
   }
-  solo_kernel<<<num_sms * per_sm, 32 * wpb, smem, s>>>(c);
+  solo_kernel<false><<<num_sms * per_sm, 32 * wpb, smem, s>>>(c);
   return cudaGetLastError();
+}
+
+// Through cudaLaunchKernel: its return value is this launch's own status.
+cudaError_t launch_solo_brute(const CellBuffers& c, int num_sms, cudaStream_t s) {
+  constexpr int wpb = 4;
+  constexpr size_t smem = sizeof(SoloCell) * wpb;
+  static_assert(smem <= 48 * 1024, "no attribute to set");
+  int blocks = (c.n + wpb - 1) / wpb;
+  if (num_sms > 0 && blocks > 4 * num_sms) blocks = 4 * num_sms;
+  CellBuffers arg = c;
+  void* args[] = {(void*)&arg};
+  return cudaLaunchKernel((const void*)solo_kernel<true>, dim3(blocks), dim3(32 * wpb), args, smem, s);
 }
 
 }  // namespace vd

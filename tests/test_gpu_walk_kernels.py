@@ -109,3 +109,27 @@ def test_cells_that_reach_far(vdmod, n):
     res = vdmod.Context(0).build(torch.from_numpy(x).cuda(), None, W.UNIT_BOX)
     cells = torch.argsort(res.volume, descending=True)[:200].cpu().numpy()
     check(res, oracle.cells(x, cells=cells), cells)
+
+
+@pytest.mark.parametrize("n", [1, 2, 31, 32, 33, 64, 65, 97, 4097, 16384])
+def test_without_a_tree(vdmod, n):
+    """vd_cells_noalloc reads the sites 64 a step, after the nearest of every 32nd."""
+    import ctypes
+
+    x = W.uniform(n, 90 + n)
+    w = W.gaussian_weights(x, 3) if n > 2 else None
+    p = lambda t: None if t is None else ctypes.c_void_p(t.data_ptr())
+    xs, ws = torch.from_numpy(x).cuda(), None if w is None else torch.from_numpy(w).cuda()
+    counts, status = (torch.full((m,), -7, dtype=torch.int32, device="cuda") for m in (n, 1))
+    nbrs = torch.full((n, 64), -7, dtype=torch.int32, device="cuda")
+    vol, cen = torch.empty(n, device="cuda"), torch.empty(n, 3, device="cuda")
+    rc = vdmod.load_library().vd_cells_noalloc(p(xs), p(ws), n, vdmod._box(W.UNIT_BOX), p(counts), p(nbrs), p(vol), p(cen),
+                                               p(status), ctypes.c_void_p(torch.cuda.current_stream().cuda_stream))
+    assert rc == vdmod.VD_OK and int(status.item()) == vdmod.VD_OK
+    cells = np.arange(n) if n < 200 else np.unique(W.rng_for(n).integers(0, n, 300))
+    ref = oracle.cells(x, w, cells=cells)
+    counts, nbrs, vol = counts.cpu().numpy(), nbrs.cpu().numpy(), vol.double().cpu().numpy()
+    for q, i in enumerate(cells):
+        assert np.array_equal(nbrs[i, :counts[i]], ref["nbrs"][q]), f"cell {i}"
+        assert np.all(nbrs[i, counts[i]:] == -7), f"cell {i}: written past its row"
+    assert np.all(np.abs(vol[cells] - ref["vol"]) <= 1e-5 * ref["vol"] + 1e-30)
