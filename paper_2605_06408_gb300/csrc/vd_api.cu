@@ -618,13 +618,17 @@ int vd_build_batched(vd_ctx* ctx, const float* xyz, const float* weights, const 
 // One pass of the adjoint kernels over the last build's cells: gradients
 // (mode 0), mesh vertex counts (1) or mesh output (2).
 static int back_pass(vd_ctx* ctx, BackBuffers b, cudaStream_t s) {
-  cudaMemsetAsync(ctx->work + 2, 0, sizeof(int) * 3, s);
+  cudaMemsetAsync(ctx->work + 2, 0, sizeof(int) * 4, s);
+  cudaMemsetAsync(ctx->work + 7, 0, sizeof(int), s);
   b.c = cell_buffers(ctx);
   b.inv_perm = ctx->inv_perm;
   b.list = ctx->blist;
   b.list_count = ctx->work + 4;
   b.list_cap = ctx->ovf_cap;
   b.work = ctx->work + 2;
+  b.list2 = ctx->mid_list;
+  b.list2_count = ctx->work + 5;
+  b.list2_next = ctx->work + 7;
   return cuda_fail(launch_backward(b, ctx->num_sms, s));
 }
 
@@ -653,7 +657,7 @@ static int backward_common(vd_ctx* ctx, const float* grad_volume, const float* g
   ctx->last_stream = s;
   ctx->ev_valid = ctx->cfg.timing != 0;
   ctx->ev_backward = true;
-  ctx->launches = 2;
+  ctx->launches = 2 + (b.tape ? 1 : 0);
   return rc;
 }
 
