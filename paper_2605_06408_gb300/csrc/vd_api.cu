@@ -35,6 +35,9 @@ struct Layout {
   }
 };
 
+// bytes before the sort's scratch: 16 ints (work counters, weight range), the status block
+constexpr size_t kClearHead = (64 + sizeof(DevStatus) + 255) & ~size_t(255);
+
 int64_t ovf_capacity(int64_t n) { return n > 4096 ? n : 4096; }
 int64_t pool_capacity(int64_t n) { return n > (1 << 22) ? n : (1 << 22); }
 int big_warps(int num_sms) { return num_sms * kBigBlocksPerSm * kBigWarpsPerBlock; }
@@ -176,7 +179,8 @@ static Layout make_layout(int64_t n, int num_sms) {
   L.add(sizeof(int) * n);              // 3 vals_a
   L.add(sizeof(int) * n);              // 4 vals_b
   L.add(sizeof(int) * n);              // 5 inv_perm
-  L.add(sort_scratch_bytes(n));        // 6 sort scratch
+  // what every build clears, in one piece: work counters and weight range, status, then the sort's scratch
+  L.add(kClearHead + sort_scratch_bytes(n));  // 6
   L.add(sizeof(int) * n);              // 7 left
   L.add(sizeof(int) * n);              // 8 right
   L.add(sizeof(int) * 2 * n);          // 9 parent
@@ -192,8 +196,8 @@ static Layout make_layout(int64_t n, int num_sms) {
   L.add(sizeof(int) * n);              // 19 ovf_slot
   L.add(sizeof(int) * ovf);            // 20 blist
   L.add(sizeof(long long) * nb);       // 21 block_sums
-  L.add(sizeof(int) * 16);             // 22 work (+ weight range)
-  L.add(sizeof(DevStatus));            // 23 status
+  L.add(0);                            // 22, 23 (with 6)
+  L.add(0);
   L.add(sizeof(SetInfo) * kMaxSets);   // 24 sets
   L.add(big_arena_bytes() * (size_t)big_warps(num_sms));  // 25 arenas
   L.add((size_t)n);                    // 26 duplicate losers
@@ -265,7 +269,10 @@ static int reserve(vd_ctx* ctx, int64_t n) {
   ctx->vals_a = (int*)(b + L.off[3]);
   ctx->vals_b = (int*)(b + L.off[4]);
   ctx->inv_perm = (int*)(b + L.off[5]);
-  ctx->hist = (unsigned*)(b + L.off[6]);
+  ctx->work = (int*)(b + L.off[6]);
+  ctx->wrange = (unsigned*)(ctx->work + 8);
+  ctx->st = (DevStatus*)(b + L.off[6] + 64);
+  ctx->hist = (unsigned*)(b + L.off[6] + kClearHead);
   ctx->left = (int*)(b + L.off[7]);
   ctx->right = (int*)(b + L.off[8]);
   ctx->parent = (int*)(b + L.off[9]);
@@ -293,9 +300,6 @@ static int reserve(vd_ctx* ctx, int64_t n) {
   ctx->ovf_slot = (int*)(b + L.off[19]);
   ctx->blist = (int*)(b + L.off[20]);
   ctx->block_sums = (long long*)(b + L.off[21]);
-  ctx->work = (int*)(b + L.off[22]);
-  ctx->wrange = (unsigned*)(ctx->work + 8);
-  ctx->st = (DevStatus*)(b + L.off[23]);
   ctx->sets_dev = (SetInfo*)(b + L.off[24]);
   reserve_tape(ctx);
   return VD_OK;
@@ -366,18 +370,15 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   mark(ctx, 0, s);
   e = cudaMemcpyAsync(ctx->sets_dev, ctx->sets_host, sizeof(SetInfo) * nsets, cudaMemcpyHostToDevice, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
-  cudaMemsetAsync(ctx->st, 0, sizeof(DevStatus), s);
-  cudaMemsetAsync(ctx->work, 0, sizeof(int) * 8, s);
+  if (cudaMemsetAsync(ctx->work, 0, kClearHead + sizeof(unsigned) * sort_clear_words(n), s) != cudaSuccess)
+    return VD_ERR_CUDA;
   if (ctx->test_stall) cudaMemsetAsync(ctx->work + 6, 1, sizeof(int), s);  // arm the test hook's token
-  cudaMemsetAsync(ctx->ovf_slot, 0xff, sizeof(int) * (size_t)n, s);
-  cudaMemsetAsync(ctx->counts, 0, sizeof(int) * (size_t)n, s);
   // 1. keys: (set, weight stratum, Morton code in the set's box); input validation
   e = launch_weight_range(w, n, ctx->sets_dev, nsets, ctx->wrange, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
-  if (launch_sort_clear(ctx->hist, n, s) != cudaSuccess) return VD_ERR_CUDA;
   const int bin_shift = nsets > 1 ? 51 : 60;
   e = launch_pack_keys(xyz, w, n, ctx->sets_dev, nsets, set_shift, bin_shift, ctx->wrange, ctx->keys_a,
-                       ctx->vals_a, ctx->hist, ctx->st, s);
+                       ctx->vals_a, ctx->hist, ctx->counts, ctx->ovf_slot, ctx->st, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
   mark(ctx, 1, s);
   // 2. radix sort of (key, index)
@@ -392,11 +393,8 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   ctx->perm = v0;
   mark(ctx, 2, s);
   // 3. packed float4 sites in Morton order (App. A.1)
-  e = launch_gather_sites(xyz, w, ctx->perm, n, ctx->sets_dev, ctx->keys_sorted, set_shift, nsets, ctx->sites, s);
-  if (e != cudaSuccess) return VD_ERR_CUDA;
-  e = launch_inverse_perm(ctx->perm, n, ctx->inv_perm, s);
-  if (e != cudaSuccess) return VD_ERR_CUDA;
-  e = launch_mark_losers(ctx->keys_sorted, ctx->sites, ctx->perm, n, ctx->loser, s);
+  e = launch_gather_sites(xyz, w, ctx->perm, n, ctx->sets_dev, ctx->keys_sorted, set_shift, nsets, ctx->sites,
+                          ctx->inv_perm, ctx->loser, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
   // 4. LBVH with per-node max weight (App. A.2)
   BvhBuffers b;
@@ -452,10 +450,9 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   ctx->last_stream = s;
   ctx->ev_valid = ctx->cfg.timing != 0;
   ctx->ev_backward = false;
-  int passes = (bits + 7) / 8;
-  ctx->launches = (w ? 1 : 0) + 1 + passes + 3 + (n >= 2 ? 4 : 1) + 2 + 3 +
-                  (out->neighbors && out->nnz_capacity > 0) + 1 + (knn ? 1 : 0) +
-                  (quad ? 1 : 0) + (uses_wide(ctx->cfg) && n >= 2);
+  const int sorts = n <= 1 ? 0 : (n <= 2048 ? 1 : (bits + 7) / 8);
+  // weights, keys, sort, sites, tree (2), records, KNN, cells (1 or 2), large cells, scan, rows
+  ctx->launches = (w ? 1 : 0) + 1 + sorts + 1 + (n >= 2 ? 2 : 0) + 1 + (knn ? 1 : 0) + (quad ? 2 : 1) + 1 + (n > 8192 ? 3 : 1) + 1;
   return VD_OK;
 }
 

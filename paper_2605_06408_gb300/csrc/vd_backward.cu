@@ -866,14 +866,4 @@ cudaError_t launch_backward(const BackBuffers& b, int num_sms, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-__global__ void inverse_perm_kernel(const int* __restrict__ perm, int n, int* __restrict__ inv) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) inv[perm[k]] = k;
-}
-
-cudaError_t launch_inverse_perm(const int* perm, int n, int* inv, cudaStream_t s) {
-  int blocks = min((n + 255) / 256, 4096);
-  inverse_perm_kernel<<<blocks, 256, 0, s>>>(perm, n, inv);
-  return cudaGetLastError();
-}
-
 }  // namespace vd

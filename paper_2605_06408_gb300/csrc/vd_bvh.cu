@@ -36,7 +36,8 @@ __device__ __forceinline__ int find_set(const SetInfo* sets, int nsets, int i) {
   return lo;
 }
 
-// Range of the weights of weighted sets (orderable-uint min / max).
+// Range of the weights of weighted sets: wr[0] the complement of the least
+// orderable value, wr[1] the greatest, so that both start at 0 (no weight).
 __global__ void weight_range_kernel(const float* __restrict__ w, int n, const SetInfo* __restrict__ sets, int nsets,
                                     unsigned* __restrict__ wr) {
   uint32_t mn = 0xffffffffu, mx = 0u;
@@ -50,15 +51,13 @@ __global__ void weight_range_kernel(const float* __restrict__ w, int n, const Se
   mn = __reduce_min_sync(FULL, mn);
   mx = __reduce_max_sync(FULL, mx);
   if ((threadIdx.x & 31) == 0) {
-    atomicMin(&wr[0], mn);
+    atomicMax(&wr[0], ~mn);
     atomicMax(&wr[1], mx);
   }
 }
 
 cudaError_t launch_weight_range(const float* w, int n, const SetInfo* sets, int nsets, unsigned* wr,
                                 cudaStream_t s) {
-  cudaMemsetAsync(wr, 0xff, sizeof(unsigned), s);
-  cudaMemsetAsync(wr + 1, 0, sizeof(unsigned), s);
   if (!w) return cudaGetLastError();
   int blocks = min((n + 255) / 256, 1024);
   weight_range_kernel<<<blocks, 256, 0, s>>>(w, n, sets, nsets, wr);
@@ -81,13 +80,15 @@ __device__ __forceinline__ uint32_t weight_bin(float w, float wmin, float wmax) 
 __global__ void pack_keys_kernel(const float* __restrict__ xyz, const float* __restrict__ w, int n,
                                  const SetInfo* __restrict__ sets, int nsets, int set_shift, int bin_shift,
                                  const unsigned* __restrict__ wr, uint64_t* __restrict__ keys, int* __restrict__ vals,
-                                 unsigned* __restrict__ hist, DevStatus* st) {
+                                 unsigned* __restrict__ hist, int* __restrict__ counts, int* __restrict__ ovf_slot,
+                                 DevStatus* st) {
   __shared__ unsigned h[8][256];  // the sort's digit counts
   for (int k = threadIdx.x; k < 8 * 256; k += blockDim.x) (&h[0][0])[k] = 0;
   __syncthreads();
   const int bits = bin_shift / 3;
   const float scale = (float)(1u << bits);
-  const float wmin = o2f(wr[0]), wmax = o2f(wr[1]);
+  const unsigned least = ~wr[0], most = wr[1];
+  const float wmin = o2f(least), wmax = o2f(most);
   for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
     float x = xyz[3 * i], y = xyz[3 * i + 1], z = xyz[3 * i + 2];
     int s = nsets > 1 ? find_set(sets, nsets, i) : 0;
@@ -105,10 +106,12 @@ __global__ void pack_keys_kernel(const float* __restrict__ xyz, const float* __r
       q[k] = (uint32_t)fminf(v, scale - 1.0f);
     }
     uint64_t code = (spread3(q[0]) << 2) | (spread3(q[1]) << 1) | spread3(q[2]);
-    uint32_t bin = (w && S.weighted && wr[0] <= wr[1]) ? weight_bin(w[i], wmin, wmax) : 0u;
+    uint32_t bin = (w && S.weighted && least <= most) ? weight_bin(w[i], wmin, wmax) : 0u;
     const uint64_t key = ((uint64_t)s << set_shift) | ((uint64_t)bin << bin_shift) | code;
     keys[i] = key;
     vals[i] = i;
+    counts[i] = 0;  // no neighbours, no place in the pool yet
+    ovf_slot[i] = -1;
 #pragma unroll
     for (int d = 0; d < 8; d++) atomicAdd(&h[d][(unsigned)(key >> (8 * d)) & 255u], 1u);
   }
@@ -120,11 +123,12 @@ __global__ void pack_keys_kernel(const float* __restrict__ xyz, const float* __r
 }
 
 cudaError_t launch_pack_keys(const float* xyz, const float* w, int n, const SetInfo* sets, int nsets, int set_shift,
-                             int bin_shift, const unsigned* wr, uint64_t* keys, int* vals, unsigned* hist, DevStatus* st,
-                             cudaStream_t s) {
+                             int bin_shift, const unsigned* wr, uint64_t* keys, int* vals, unsigned* hist, int* counts,
+                             int* ovf_slot, DevStatus* st, cudaStream_t s) {
   int threads = 256;
   int blocks = min((n + threads - 1) / threads, 1024);
-  pack_keys_kernel<<<blocks, threads, 0, s>>>(xyz, w, n, sets, nsets, set_shift, bin_shift, wr, keys, vals, hist, st);
+  pack_keys_kernel<<<blocks, threads, 0, s>>>(xyz, w, n, sets, nsets, set_shift, bin_shift, wr, keys, vals, hist, counts, ovf_slot,
+                                              st);
   return cudaGetLastError();
 }
 
@@ -282,14 +286,104 @@ size_t sort_scratch_bytes(int64_t n) {
   return sizeof(unsigned) * (kSortHist + 2 * 256 * (size_t)tiles);
 }
 
-// Clear the digit counts that the keys' kernel adds to, the tickets and the first chain.
-cudaError_t launch_sort_clear(unsigned* scratch, int n, cudaStream_t s) {
-  return cudaMemsetAsync(scratch, 0, sizeof(unsigned) * (kSortHist + 256 * (size_t)sort_tiles(n)), s);
+// Words at the head of the scratch that must start at 0: the digit counts that
+// the keys' kernel adds to, the tickets and the first chain.
+size_t sort_clear_words(int n) { return kSortHist + 256 * (size_t)sort_tiles(n); }
+
+// All digits of at most kSortSmall keys in one block: 500 keys 29 -> 14 us (and
+// seven launches less).
+constexpr int kSortSmall = 2048;
+__global__ void __launch_bounds__(512) sort_small_kernel(uint64_t* __restrict__ keys, int* __restrict__ vals, int n,
+                                                         int bits) {
+  constexpr int ITEMS = kSortSmall / 512, W = 16;
+  __shared__ unsigned wh[W][256];
+  __shared__ unsigned part[8];
+  __shared__ uint64_t sk[kSortSmall];
+  __shared__ int sv[kSortSmall];
+  const int t = (int)threadIdx.x, lane = t & 31, w = t >> 5;
+  const int base = w * 32 * ITEMS + lane;
+  uint64_t key[ITEMS];
+  int val[ITEMS], rank[ITEMS];
+#pragma unroll
+  for (int i = 0; i < ITEMS; i++) {
+    const int at = base + 32 * i;
+    key[i] = at < n ? keys[at] : ~0ull;
+    val[i] = at < n ? vals[at] : 0;
+  }
+  for (int shift = 0; shift < bits; shift += 8) {
+    for (int k = t; k < W * 256; k += 512) (&wh[0][0])[k] = 0;
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+      const bool in = base + 32 * i < n;
+      const unsigned d = in ? (unsigned)(key[i] >> shift) & 255u : 256u;
+      const unsigned peers = __match_any_sync(FULL, d);
+      const unsigned before = in ? wh[w][d] : 0u;
+      rank[i] = (int)before + __popc(peers & lanemask_lt());
+      __syncwarp();
+      if (in && (peers >> lane) == 1u) wh[w][d] = before + __popc(peers);
+      __syncwarp();
+    }
+    __syncthreads();
+    unsigned count = 0, a = 0;
+    if (t < 256) {
+#pragma unroll
+      for (int q = 0; q < W; q++) {
+        const unsigned c = wh[q][t];
+        wh[q][t] = count;
+        count += c;
+      }
+      a = count;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const unsigned x = __shfl_up_sync(FULL, a, o);
+        if (lane >= o) a += x;
+      }
+      if (lane == 31) part[w] = a;
+    }
+    __syncthreads();
+    if (t < 256) {
+      a -= count;
+      for (int q = 0; q < w; q++) a += part[q];
+#pragma unroll
+      for (int q = 0; q < W; q++) wh[q][t] += a;
+    }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++)
+      if (base + 32 * i < n) {
+        const int to = rank[i] + (int)wh[w][(unsigned)(key[i] >> shift) & 255u];
+        sk[to] = key[i];
+        sv[to] = val[i];
+      }
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < ITEMS; i++) {
+      const int at = base + 32 * i;
+      if (at < n) {
+        key[i] = sk[at];
+        val[i] = sv[at];
+      }
+    }
+    __syncthreads();
+  }
+#pragma unroll
+  for (int i = 0; i < ITEMS; i++) {
+    const int at = base + 32 * i;
+    if (at < n) {
+      keys[at] = key[i];
+      vals[at] = val[i];
+    }
+  }
 }
 
 cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, int*& vals_alt, unsigned* scratch, int n,
                              int bits, DevStatus* st, cudaStream_t s) {
   if (n <= 1) return cudaSuccess;
+  if (n <= kSortSmall) {
+    sort_small_kernel<<<1, 512, 0, s>>>(keys, vals, n, bits);
+    return cudaGetLastError();
+  }
   const int tiles = sort_tiles(n);
   unsigned* chain = scratch + kSortHist;
   unsigned* other = chain + 256 * (size_t)tiles;
@@ -308,52 +402,45 @@ cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, i
 }
 
 // ---------------------------------------------------------------- packed sorted sites
-
+//
+// The packed site of every sorted place, the inverse permutation, and the
+// losers of duplicate positions: sites at exactly the same position (and
+// weight stratum) share a key and are adjacent after the sort. Among them the
+// larger weight, then the lower original index, keeps its cell; every other
+// one has an empty cell, and its half-space is implied by the winner's, so it
+// is never a candidate.
 __global__ void gather_sites_kernel(const float* __restrict__ xyz, const float* __restrict__ w,
                                     const int* __restrict__ perm, int n, const SetInfo* __restrict__ sets,
                                     const uint64_t* __restrict__ keys, int set_shift, int nsets,
-                                    float4* __restrict__ sites) {
+                                    float4* __restrict__ sites, int* __restrict__ inv,
+                                    unsigned char* __restrict__ loser) {
   for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    int i = perm[k];
-    int s = nsets > 1 ? (int)(keys[k] >> set_shift) : 0;
-    float wi = (w && sets[s].weighted) ? w[i] : 0.0f;
-    sites[k] = make_float4(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], wi);
-  }
-}
-
-cudaError_t launch_gather_sites(const float* xyz, const float* w, const int* perm, int n, const SetInfo* sets,
-                                const uint64_t* keys, int set_shift, int nsets, float4* sites, cudaStream_t s) {
-  int threads = 256;
-  int blocks = min((n + threads - 1) / threads, 4096);
-  gather_sites_kernel<<<blocks, threads, 0, s>>>(xyz, w, perm, n, sets, keys, set_shift, nsets, sites);
-  return cudaGetLastError();
-}
-
-// ---------------------------------------------------------------- duplicates
-// Sites at exactly the same position share a Morton key and are adjacent
-// after the sort. Among them the larger weight, then the lower original
-// index, keeps its cell; every other one has an empty cell, and its
-// half-space is implied by the winner's, so it is never a candidate.
-__global__ void mark_losers_kernel(const uint64_t* __restrict__ keys, const float4* __restrict__ sites,
-                                   const int* __restrict__ perm, int n, unsigned char* __restrict__ loser) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    uint64_t key = keys[k];
-    float4 p = sites[k];
+    const int i = perm[k];
+    const uint64_t key = keys[k];
+    const int s = nsets > 1 ? (int)(key >> set_shift) : 0;
+    const bool weighted = w && sets[s].weighted;
+    const float4 p = make_float4(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], weighted ? w[i] : 0.0f);
+    sites[k] = p;
+    inv[i] = k;
     bool lose = false;
     for (int dir = -1; dir <= 1 && !lose; dir += 2)
       for (int m = k + dir; m >= 0 && m < n && keys[m] == key && !lose; m += dir) {
-        float4 q = sites[m];
-        if (q.x == p.x && q.y == p.y && q.z == p.z)
-          lose = q.w > p.w || (q.w == p.w && perm[m] < perm[k]);
+        const int o = perm[m];
+        if (xyz[3 * o] == p.x && xyz[3 * o + 1] == p.y && xyz[3 * o + 2] == p.z) {
+          const float qw = weighted ? w[o] : 0.0f;
+          lose = qw > p.w || (qw == p.w && o < i);
+        }
       }
     loser[k] = lose ? 1 : 0;
   }
 }
 
-cudaError_t launch_mark_losers(const uint64_t* keys, const float4* sites, const int* perm, int n,
-                               unsigned char* loser, cudaStream_t s) {
-  int blocks = min((n + 255) / 256, 4096);
-  mark_losers_kernel<<<blocks, 256, 0, s>>>(keys, sites, perm, n, loser);
+cudaError_t launch_gather_sites(const float* xyz, const float* w, const int* perm, int n, const SetInfo* sets,
+                                const uint64_t* keys, int set_shift, int nsets, float4* sites, int* inv,
+                                unsigned char* loser, cudaStream_t s) {
+  int threads = 256;
+  int blocks = min((n + threads - 1) / threads, 4096);
+  gather_sites_kernel<<<blocks, threads, 0, s>>>(xyz, w, perm, n, sets, keys, set_shift, nsets, sites, inv, loser);
   return cudaGetLastError();
 }
 
@@ -369,9 +456,11 @@ __device__ __forceinline__ int common_prefix(const uint64_t* keys, int n, int i,
 // Internal node i of the binary radix tree over n sorted keys (ties broken
 // by position). Children: internal index >= 0, or -1-site for a single site.
 __global__ void karras_kernel(const uint64_t* __restrict__ keys, int n, int* __restrict__ left,
-                              int* __restrict__ right, int* __restrict__ parent, int2* __restrict__ range) {
+                              int* __restrict__ right, int* __restrict__ parent, int2* __restrict__ range,
+                              int* __restrict__ visit) {
   int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n - 1) return;
+  visit[i] = 0;
   int dplus = common_prefix(keys, n, i, i + 1), dminus = common_prefix(keys, n, i, i - 1);
   int d = dplus > dminus ? 1 : -1;
   int dmin = min(dplus, dminus);
@@ -436,51 +525,39 @@ __global__ void refit_kernel(const float4* __restrict__ sites, const int* __rest
   }
 }
 
-// Traversal record of internal node i: both children's boxes, max weights
-// and references (64 bytes, read by four lanes with one float4 each).
-__global__ void emit_nodes_kernel(const float4* __restrict__ sites, const int* __restrict__ left,
-                                  const int* __restrict__ right, const int2* __restrict__ range,
-                                  const float4* __restrict__ box_lo, const float4* __restrict__ box_hi, int n,
-                                  int leaf_size, float4* __restrict__ nodes) {
-  int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n - 1) return;
-#pragma unroll
-  for (int c = 0; c < 2; c++) {
-    int ch = c == 0 ? left[i] : right[i];
-    float4 lo, hi;
-    int ref;
-    if (ch < 0) {
-      float4 p = sites[-1 - ch];
-      lo = p;
-      hi = make_float4(p.x, p.y, p.z, 0.0f);
-      ref = make_leaf_ref(-1 - ch, 1);
-    } else {
-      lo = box_lo[ch];
-      hi = box_hi[ch];
-      int2 r = range[ch];
-      int cnt = r.y - r.x + 1;
-      ref = cnt <= leaf_size ? make_leaf_ref(r.x, cnt) : ch;
-    }
-    hi.w = __int_as_float(ref);
-    nodes[4 * i + 2 * c] = lo;
-    nodes[4 * i + 2 * c + 1] = hi;
-  }
-}
-
 // 8-wide traversal record of internal node i: the nodes three binary levels
 // below it, or the leaf (at most kWideLeaf sites) a path ends at earlier, in
 // the slot of that path followed by zeros; the other slots are empty. Eight
 // boxes' low corners (w: maximum weight), then their high corners (w:
 // reference), so that eight lanes read each half as one 128-byte line.
-__global__ void emit_wide_kernel(const float4* __restrict__ sites, const int* __restrict__ left,
-                                 const int* __restrict__ right, const int2* __restrict__ range,
-                                 const float4* __restrict__ box_lo, const float4* __restrict__ box_hi, int n,
-                                 float4* __restrict__ wide) {
-  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-  const int i = (int)(tid >> 3), s = (int)(tid & 7);
-  if (i >= n - 1) return;
+// The binary record (both children's boxes, max weights and references: 64
+// bytes, read by four lanes with one float4 each) by the first two of the
+// eight threads.
+__device__ __forceinline__ void emit_node(int i, int s, const float4* __restrict__ sites, const int* __restrict__ left,
+                                          const int* __restrict__ right, const int2* __restrict__ range,
+                                          const float4* __restrict__ box_lo, const float4* __restrict__ box_hi,
+                                          int leaf_size, float4* __restrict__ nodes, float4* __restrict__ wide) {
+  if (s < 2) {
+    const int ch = s == 0 ? left[i] : right[i];
+    float4 lo, hi;
+    int ref;
+    if (ch < 0) {
+      lo = sites[-1 - ch];
+      hi = lo;
+      ref = make_leaf_ref(-1 - ch, 1);
+    } else {
+      lo = box_lo[ch];
+      hi = box_hi[ch];
+      const int2 r = range[ch];
+      const int cnt = r.y - r.x + 1;
+      ref = cnt <= leaf_size ? make_leaf_ref(r.x, cnt) : ch;
+    }
+    hi.w = __int_as_float(ref);
+    nodes[4 * (size_t)i + 2 * s] = lo;
+    nodes[4 * (size_t)i + 2 * s + 1] = hi;
+  }
   const int2 own = range[i];
-  if (own.y - own.x < kWideLeaf) return;  // inside a leaf: never visited
+  if (!wide || own.y - own.x < kWideLeaf) return;  // inside a leaf: never visited
   int c = i, first = own.x, cnt = own.y - own.x + 1;
   bool valid = true;
 #pragma unroll
@@ -517,10 +594,8 @@ __global__ void emit_wide_kernel(const float4* __restrict__ sites, const int* __
 }
 
 // Root references of every set: the node whose range is exactly the set.
-__global__ void set_roots_kernel(SetInfo* sets, int nsets, const int2* __restrict__ range, int n, int leaf_size,
-                                 DevStatus* st) {
-  int s = blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= nsets) return;
+__device__ __forceinline__ void set_root(SetInfo* sets, int s, const int2* __restrict__ range, int n, int leaf_size,
+                                         DevStatus* st) {
   int f = sets[s].first, c = sets[s].count;
   if (c <= 0) {
     sets[s].root = sets[s].wroot = 0;
@@ -543,22 +618,30 @@ __global__ void set_roots_kernel(SetInfo* sets, int nsets, const int2* __restric
   sets[s].wroot = c <= kWideLeaf ? make_leaf_ref(f, c) : node;
 }
 
+// The traversal records, and the sets' roots.
+__global__ void emit_kernel(const float4* __restrict__ sites, const int* __restrict__ left,
+                            const int* __restrict__ right, const int2* __restrict__ range,
+                            const float4* __restrict__ box_lo, const float4* __restrict__ box_hi, int n, int leaf_size,
+                            float4* __restrict__ nodes, float4* __restrict__ wide, SetInfo* sets, int nsets,
+                            DevStatus* st) {
+  const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (tid < nsets) set_root(sets, (int)tid, range, n, leaf_size, st);
+  const int i = (int)(tid >> 3);
+  if (i < n - 1) emit_node(i, (int)(tid & 7), sites, left, right, range, box_lo, box_hi, leaf_size, nodes, wide);
+}
+
 cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, int leaf_size, BvhBuffers& b,
                              SetInfo* sets, int nsets, DevStatus* st, cudaStream_t s) {
   int threads = 256;
   if (n >= 2) {
     int blocks = (n - 1 + threads - 1) / threads;
-    karras_kernel<<<blocks, threads, 0, s>>>(keys, n, b.left, b.right, b.parent, b.range);
-    cudaMemsetAsync(b.visit, 0, sizeof(int) * (size_t)(n - 1), s);
+    karras_kernel<<<blocks, threads, 0, s>>>(keys, n, b.left, b.right, b.parent, b.range, b.visit);
     refit_kernel<<<(n + threads - 1) / threads, threads, 0, s>>>(sites, b.left, b.right, b.parent, b.visit,
                                                                   b.box_lo, b.box_hi, n);
-    emit_nodes_kernel<<<blocks, threads, 0, s>>>(sites, b.left, b.right, b.range, b.box_lo, b.box_hi, n, leaf_size,
-                                                 b.nodes);
-    if (b.wide)
-      emit_wide_kernel<<<(int)((8ll * (n - 1) + threads - 1) / threads), threads, 0, s>>>(
-          sites, b.left, b.right, b.range, b.box_lo, b.box_hi, n, b.wide);
   }
-  set_roots_kernel<<<(nsets + 127) / 128, 128, 0, s>>>(sets, nsets, b.range, n, leaf_size, st);
+  const long long work = std::max<long long>(8ll * (n - 1), nsets);
+  emit_kernel<<<(int)((work + threads - 1) / threads), threads, 0, s>>>(sites, b.left, b.right, b.range, b.box_lo, b.box_hi,
+                                                                       n, leaf_size, b.nodes, b.wide, sets, nsets, st);
   return cudaGetLastError();
 }
 

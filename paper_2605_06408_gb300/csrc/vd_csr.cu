@@ -91,14 +91,26 @@ __global__ void __launch_bounds__(kScanThreads) scan_write_kernel(const int* __r
   if (base + kScanItems >= n && base < n) offsets[n] = (int)*total;
 }
 
+// The status and the total after the rows: once per call.
+__device__ __forceinline__ void finish_status(DevStatus* st, long long nnz, long long cap, int64_t* nnz_out,
+                                              int32_t* user_status) {
+  if (nnz > cap)
+    set_error(st, VD_ERR_CAPACITY);
+  else
+    atomicCAS(&st->error, VD_ERR_CAPACITY, 0);  // a re-copy into a large enough buffer
+  if (nnz_out) *nnz_out = nnz;
+  if (user_status) *user_status = st->error;
+}
+
 // one warp per row: copy the row's neighbours from its scratch row (or the
-// large-cell pool)
+// large-cell pool); the first thread finishes the call's status
 __global__ void compact_kernel(const int* __restrict__ counts, const int* __restrict__ offsets,
                                const int* __restrict__ scratch, int stride, const int* __restrict__ pool,
                                const int* __restrict__ ovf_slot, int n, int* __restrict__ nbrs,
-                               long long cap, const DevStatus* st) {
-  long long nnz = st->nnz;
-  if (nnz > cap || nnz > 0x7fffffffLL) return;
+                               long long cap, DevStatus* st, int64_t* nnz_out, int32_t* user_status) {
+  const long long nnz = st->nnz;
+  if (blockIdx.x == 0 && threadIdx.x == 0) finish_status(st, nnz, nbrs ? cap : 0x7fffffffffffffffLL, nnz_out, user_status);
+  if (!nbrs || nnz > cap || nnz > 0x7fffffffLL) return;
   const int lane = threadIdx.x & 31;
   const int warps = gridDim.x * (blockDim.x >> 5);
   for (int row = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); row < n; row += warps) {
@@ -111,32 +123,43 @@ __global__ void compact_kernel(const int* __restrict__ counts, const int* __rest
   }
 }
 
-__global__ void finish_status_kernel(DevStatus* st, long long cap, int64_t* nnz_out, int32_t* user_status) {
-  long long nnz = st->nnz;
-  if (nnz > cap)
-    set_error(st, VD_ERR_CAPACITY);
-  else
-    atomicCAS(&st->error, VD_ERR_CAPACITY, 0);  // a re-copy into a large enough buffer
-  if (nnz_out) *nnz_out = nnz;
-  if (user_status) *user_status = st->error;
+// Exclusive scan of at most one tile of counts in one launch.
+__global__ void __launch_bounds__(kScanThreads) scan_tile_kernel(const int* __restrict__ counts, int n,
+                                                                 int* __restrict__ offsets, long long* __restrict__ total) {
+  __shared__ long long wt[32];
+  const int base = threadIdx.x * kScanItems;
+  int c[kScanItems];
+  long long s = 0;
+#pragma unroll
+  for (int k = 0; k < kScanItems; k++) {
+    c[k] = base + k < n ? counts[base + k] : 0;
+    s += c[k];
+  }
+  const long long inc = block_inclusive_scan(s, wt);
+  long long run = inc - s;
+#pragma unroll
+  for (int k = 0; k < kScanItems; k++) {
+    if (base + k < n) offsets[base + k] = (int)run;
+    run += c[k];
+  }
+  if (threadIdx.x == kScanThreads - 1) {
+    offsets[n] = (int)inc;
+    *total = inc;
+  }
 }
 
 cudaError_t launch_csr(const CellBuffers& c, int32_t* offsets, int32_t* neighbors, int64_t cap, int64_t* nnz_out,
                        long long* block_sums, int32_t* user_status, bool recount, cudaStream_t s) {
   int n = c.n;
-  int nb = (n + kScanTile - 1) / kScanTile;
   if (recount) {
-    scan_reduce_kernel<<<nb, kScanThreads, 0, s>>>(c.counts, n, block_sums);
-    scan_bsum_kernel<<<1, kScanThreads, 0, s>>>(block_sums, nb, &c.st->nnz, c.st);
-    scan_write_kernel<<<nb, kScanThreads, 0, s>>>(c.counts, n, block_sums, offsets, &c.st->nnz);
+    cudaError_t e = launch_scan(c.counts, n, offsets, block_sums, &c.st->nnz, c.st, s);
+    if (e != cudaSuccess) return e;
   }
-  if (neighbors && cap > 0) {
-    int blocks = (n + 7) / 8;
-    if (blocks > 65536) blocks = 65536;
-    compact_kernel<<<blocks, 256, 0, s>>>(c.counts, offsets, c.scratch, c.stride, c.pool, c.ovf_slot, n,
-                                          neighbors, neighbors ? cap : 0, c.st);
-  }
-  finish_status_kernel<<<1, 1, 0, s>>>(c.st, neighbors ? cap : 0x7fffffffffffffffLL, nnz_out, user_status);
+  const bool rows = neighbors && cap > 0;
+  int blocks = rows ? (n + 7) / 8 : 1;
+  if (blocks > 65536) blocks = 65536;
+  compact_kernel<<<blocks, 256, 0, s>>>(c.counts, offsets, c.scratch, c.stride, c.pool, c.ovf_slot, n,
+                                        neighbors, cap, c.st, nnz_out, user_status);
   return cudaGetLastError();
 }
 
@@ -154,6 +177,10 @@ cudaError_t launch_mesh_finish(const DevStatus* st, int64_t* nverts_out, int32_t
 cudaError_t launch_scan(const int* counts, int n, int32_t* offsets, long long* block_sums, long long* total,
                         DevStatus* st, cudaStream_t s) {
   int nb = (n + kScanTile - 1) / kScanTile;
+  if (nb == 1) {  // no total over 2^31 to watch for
+    scan_tile_kernel<<<1, kScanThreads, 0, s>>>(counts, n, offsets, total);
+    return cudaGetLastError();
+  }
   scan_reduce_kernel<<<nb, kScanThreads, 0, s>>>(counts, n, block_sums);
   scan_bsum_kernel<<<1, kScanThreads, 0, s>>>(block_sums, nb, total, st);
   scan_write_kernel<<<nb, kScanThreads, 0, s>>>(counts, n, block_sums, offsets, total);

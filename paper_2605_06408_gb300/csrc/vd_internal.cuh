@@ -346,14 +346,15 @@ struct BackBuffers {
 cudaError_t launch_weight_range(const float* w, int n, const SetInfo* sets, int nsets, unsigned* wr,
                                 cudaStream_t s);
 cudaError_t launch_pack_keys(const float* xyz, const float* w, int n, const SetInfo* sets, int nsets, int set_shift,
-                             int bin_shift, const unsigned* wr, uint64_t* keys, int* vals, unsigned* hist, DevStatus* st,
-                             cudaStream_t s);
+                             int bin_shift, const unsigned* wr, uint64_t* keys, int* vals, unsigned* hist, int* counts,
+                             int* ovf_slot, DevStatus* st, cudaStream_t s);
 size_t sort_scratch_bytes(int64_t n);
-cudaError_t launch_sort_clear(unsigned* scratch, int n, cudaStream_t s);
+size_t sort_clear_words(int n);
 cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, int*& vals_alt, unsigned* scratch, int n,
                              int bits, DevStatus* st, cudaStream_t s);
 cudaError_t launch_gather_sites(const float* xyz, const float* w, const int* perm, int n, const SetInfo* sets,
-                                const uint64_t* keys, int set_shift, int nsets, float4* sites, cudaStream_t s);
+                                const uint64_t* keys, int set_shift, int nsets, float4* sites, int* inv,
+                                unsigned char* loser, cudaStream_t s);
 cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, int leaf_size, BvhBuffers& b,
                              SetInfo* sets, int nsets, DevStatus* st, cudaStream_t s);
 cudaError_t launch_cells(const CellBuffers& c, int num_sms, cudaStream_t s, const std::function<void()>& between);
@@ -370,8 +371,5 @@ cudaError_t launch_backward(const BackBuffers& b, int num_sms, cudaStream_t s);
 cudaError_t launch_scan(const int* counts, int n, int32_t* offsets, long long* block_sums, long long* total,
                         DevStatus* st, cudaStream_t s);
 cudaError_t launch_mesh_finish(const DevStatus* st, int64_t* nverts_out, int32_t* user_status, cudaStream_t s);
-cudaError_t launch_inverse_perm(const int* perm, int n, int* inv, cudaStream_t s);
-cudaError_t launch_mark_losers(const uint64_t* keys, const float4* sites, const int* perm, int n,
-                               unsigned char* loser, cudaStream_t s);
 
 }  // namespace vd
