@@ -618,6 +618,42 @@ __device__ __forceinline__ void set_root(SetInfo* sets, int s, const int2* __res
   sets[s].wroot = c <= kWideLeaf ? make_leaf_ref(f, c) : node;
 }
 
+// The same boxes for small inputs, without the climb's chain of fences and
+// round trips (500 sites 22 us, 10,000 32 us): each node reads all of its sites.
+__global__ void __launch_bounds__(128) node_boxes_kernel(const float4* __restrict__ sites, const int2* __restrict__ range,
+                                                         float4* __restrict__ box_lo, float4* __restrict__ box_hi) {
+  __shared__ float part[7][4];
+  const int2 r = range[blockIdx.x];
+  const int t = (int)threadIdx.x;
+  float v[7];  // low corner, negated high corner, negated weight
+#pragma unroll
+  for (int k = 0; k < 7; k++) v[k] = INFINITY;
+#pragma unroll 4
+  for (int j = r.x + t; j <= r.y; j += 128) {
+    const float4 p = sites[j];
+    v[0] = fminf(v[0], p.x);
+    v[1] = fminf(v[1], p.y);
+    v[2] = fminf(v[2], p.z);
+    v[3] = fminf(v[3], -p.x);
+    v[4] = fminf(v[4], -p.y);
+    v[5] = fminf(v[5], -p.z);
+    v[6] = fminf(v[6], -p.w);
+  }
+#pragma unroll
+  for (int k = 0; k < 7; k++) {
+    for (int o = 16; o > 0; o >>= 1) v[k] = fminf(v[k], __shfl_xor_sync(FULL, v[k], o));
+    if ((t & 31) == 0) part[k][t >> 5] = v[k];
+  }
+  __syncthreads();
+  if (t == 0) {
+#pragma unroll
+    for (int k = 0; k < 7; k++) v[k] = fminf(fminf(part[k][0], part[k][1]), fminf(part[k][2], part[k][3]));
+    box_lo[blockIdx.x] = make_float4(v[0], v[1], v[2], -v[6]);
+    box_hi[blockIdx.x] = make_float4(-v[3], -v[4], -v[5], 0.0f);
+  }
+}
+constexpr int kBoxesDirect = 16384;
+
 // The traversal records, and the sets' roots.
 __global__ void emit_kernel(const float4* __restrict__ sites, const int* __restrict__ left,
                             const int* __restrict__ right, const int2* __restrict__ range,
@@ -636,8 +672,11 @@ cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, i
   if (n >= 2) {
     int blocks = (n - 1 + threads - 1) / threads;
     karras_kernel<<<blocks, threads, 0, s>>>(keys, n, b.left, b.right, b.parent, b.range, b.visit);
-    refit_kernel<<<(n + threads - 1) / threads, threads, 0, s>>>(sites, b.left, b.right, b.parent, b.visit,
-                                                                  b.box_lo, b.box_hi, n);
+    if (n <= kBoxesDirect)
+      node_boxes_kernel<<<n - 1, 128, 0, s>>>(sites, b.range, b.box_lo, b.box_hi);
+    else
+      refit_kernel<<<(n + threads - 1) / threads, threads, 0, s>>>(sites, b.left, b.right, b.parent, b.visit,
+                                                                    b.box_lo, b.box_hi, n);
   }
   const long long work = std::max<long long>(8ll * (n - 1), nsets);
   emit_kernel<<<(int)((work + threads - 1) / threads), threads, 0, s>>>(sites, b.left, b.right, b.range, b.box_lo, b.box_hi,
