@@ -317,32 +317,36 @@ class Context:
         out = {
             "offsets": torch.empty(n + 1, dtype=torch.int32, device=dev),
             "neighbors": torch.empty(max(cap, 1), dtype=torch.int32, device=dev),
-            "nnz": torch.zeros(1, dtype=torch.int64, device=dev),
+            # nnz, then the status word in the low half: written by every build, read back in one copy
+            "tail": torch.empty(2, dtype=torch.int64, device=dev),
             "volume": torch.empty(n, dtype=torch.float32, device=dev),
             "centroid": torch.empty(n, 3, dtype=torch.float32, device=dev),
-            "status": torch.zeros(1, dtype=torch.int32, device=dev),
         }
         s = VdOut()
         s.offsets = out["offsets"].data_ptr()
         s.neighbors = out["neighbors"].data_ptr()
         s.nnz_capacity = cap
-        s.nnz_out = out["nnz"].data_ptr()
+        s.nnz_out = out["tail"].data_ptr()
         s.volume = out["volume"].data_ptr()
         s.centroid = out["centroid"].data_ptr()
-        s.status = out["status"].data_ptr()
+        s.status = out["tail"].data_ptr() + 8
         return out, s
+
+    @staticmethod
+    def _read_tail(out):
+        nnz, word = out["tail"].tolist()
+        return nnz, ((word & 0xFFFFFFFF) ^ 0x80000000) - 0x80000000
 
     def _finish(self, out, s, n: int, sync: bool) -> Cells:
         if not sync:
             return Cells(out["offsets"], out["neighbors"], out["volume"], out["centroid"], 0, -1)
-        st = int(out["status"].item())
-        nnz = int(out["nnz"].item())
+        nnz, st = self._read_tail(out)
         if st == VD_ERR_CAPACITY:
             out2, s2 = self._alloc_out(n, nnz)
             out2["volume"], out2["centroid"] = out["volume"], out["centroid"]
             _check(self._lib.vd_copy_neighbors(self._h, ctypes.byref(s2), _stream_ptr(self.device)),
                    "vd_copy_neighbors")
-            st = int(out2["status"].item())
+            st = self._read_tail(out2)[1]
             out = out2
         if st != VD_OK:
             raise VdError(st, "device status")
@@ -404,24 +408,21 @@ class Context:
         n = self._last_n
         dev = self.device
         off = torch.empty(n + 1, dtype=torch.int32, device=dev)
-        nv = torch.zeros(1, dtype=torch.int64, device=dev)
-        st = torch.zeros(1, dtype=torch.int32, device=dev)
+        tail = torch.empty(2, dtype=torch.int64, device=dev)  # vertex count, status word (as in build)
         cap = int(capacity) if capacity is not None else 64 * n
 
         def run(cap):
             verts = torch.empty(max(cap, 1), 3, dtype=torch.float32, device=dev)
             sites = torch.empty(max(cap, 1), 3, dtype=torch.int32, device=dev)
-            m = VdMesh(off.data_ptr(), verts.data_ptr(), sites.data_ptr(), cap, nv.data_ptr(), st.data_ptr())
+            m = VdMesh(off.data_ptr(), verts.data_ptr(), sites.data_ptr(), cap, tail.data_ptr(), tail.data_ptr() + 8)
             _check(self._lib.vd_cells_mesh(self._h, ctypes.byref(m), _stream_ptr(dev)), "vd_cells_mesh")
-            torch.cuda.synchronize(dev)
-            return verts, sites
+            return verts, sites, *self._read_tail({"tail": tail})
 
-        verts, sites = run(cap)
-        total = int(nv.item())
-        if int(st.item()) == VD_ERR_CAPACITY or total > cap:
-            verts, sites = run(total)
-        elif int(st.item()) != VD_OK:
-            raise VdError(int(st.item()), "vd_cells_mesh")
+        verts, sites, total, st = run(cap)
+        if st == VD_ERR_CAPACITY or total > cap:
+            verts, sites, total, st = run(total)
+        elif st != VD_OK:
+            raise VdError(st, "vd_cells_mesh")
         return off, verts[:total], sites[:total]
 
     def backward(self, grad_volume: Optional[torch.Tensor], grad_centroid: Optional[torch.Tensor],
