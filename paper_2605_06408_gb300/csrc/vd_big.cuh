@@ -520,7 +520,8 @@ __device__ inline uint32_t filter_chunks(const float4* vp, const float4* cb, int
 // closes the request once every chunk is done. A claim succeeds only while
 // its generation is open and chunks remain, and the owner cannot close
 // before every claimed group is counted, so a helper never works on a
-// request that was closed or re-opened under it. Waits are bounded: a wait
+// request that was closed or re-opened under it (a closed request's counter
+// stands past any number of chunks). Waits are bounded: a wait
 // that runs out sets VD_ERR_TIMEOUT and returns.
 struct HelpReq {
   int seq;        // odd while open
@@ -642,7 +643,14 @@ __device__ inline uint32_t big_filter(const BigCell& c, const BigArena& A, int k
     __syncwarp();
     cuts = (uint32_t)vload((const int*)&r.cuts);
     cuts = __shfl_sync(FULL, cuts, 0);
-    if (lane == 0) atomicAdd(&r.seq, 1);
+    if (lane == 0) {
+      // closed for claims before the fields change: a helper that still holds
+      // this generation would else claim past the old end once a larger nch is
+      // posted, and its count would go to the next request
+      atomicExch(&r.next, (gen << 20) | 0xfffff);
+      __threadfence_block();
+      atomicAdd(&r.seq, 1);
+    }
     __syncwarp();
   }
   if (counters) ct.vtests += tested;
