@@ -212,6 +212,12 @@ __device__ __forceinline__ bool ambiguous(T s, T ev, T eh) {
   return fabs(s) <= (ev + eh) * (T(1) + T(4) * Num<T>::u);
 }
 
+// Is the site finite? One that is not (the build reports it) culls nothing, so
+// its cell would walk the whole tree: the kernels leave it empty instead.
+__device__ __forceinline__ bool finite_site(const float4& p) {
+  return isfinite(p.x) && isfinite(p.y) && isfinite(p.z) && isfinite(p.w);
+}
+
 // ---------------------------------------------------------------- warp helpers
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 __device__ __forceinline__ unsigned lanemask_lt() {

@@ -55,9 +55,11 @@ __global__ void __launch_bounds__(128) knn_kernel(const float4* __restrict__ sit
   const unsigned gsh = lane & 24u;
   const uint32_t ltg = (1u << gl) - 1u;
   const int want = begin + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 3);
-  const bool live = want < end;
-  const int si = live ? want : end - 1;
+  const int si = min(want, end - 1);
   const float4 p = sites[si];
+  // a loser of a duplicate position and a site that is not finite need no list
+  // (and would find no bound to stop at)
+  const bool own = want < end, live = own && loser[si] == 0 && finite_site(p);
   const SetInfo& SI = sets[nsets > 1 ? (int)(keys[si] >> set_shift) : 0];
   const int lo = SI.first, hi = SI.first + SI.count;
   const int w0 = max(lo, min(si - 4, hi - 9)), w1 = min(hi, w0 + 9);
@@ -182,7 +184,7 @@ __global__ void __launch_bounds__(128) knn_kernel(const float4* __restrict__ sit
       }
     }
   }
-  if (live) knn[(size_t)si * kKnn + gl] = bi;
+  if (own) knn[(size_t)si * kKnn + gl] = live ? bi : -1;
 }
 
 }  // namespace

@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
     const SetInfo& SI = P.sets[P.nsets > 1 ? (int)(P.keys[si] >> P.set_shift) : 0];
     const float* box = SI.lo;
     // a site that an exact duplicate beats has an empty cell
-    int mode = !exists ? M_IDLE : (P.loser[si] ? M_EMPTY : M_BUILD);
+    int mode = !exists ? M_IDLE : (P.loser[si] || !finite_site(me) ? M_EMPTY : M_BUILD);
     const unsigned amb0 = ctamb;
 
     // ---- the box: 6 planes, 8 corners (as init_cell)

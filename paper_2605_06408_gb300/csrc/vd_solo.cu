@@ -325,7 +325,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
     const SetInfo& SI = P.sets[P.nsets > 1 ? (int)(P.keys[si] >> P.set_shift) : 0];
     const float* box = SI.lo;
     const bool weighted = SI.weighted != 0;
-    int mode = P.loser[si] ? S_EMPTY : S_BUILD;
+    int mode = P.loser[si] || !finite_site(me) ? S_EMPTY : S_BUILD;
     const unsigned amb0 = ctamb;
 
     // ---- the box: 6 planes, 8 corners (as init_cell)

@@ -133,3 +133,24 @@ def test_without_a_tree(vdmod, n):
         assert np.array_equal(nbrs[i, :counts[i]], ref["nbrs"][q]), f"cell {i}"
         assert np.all(nbrs[i, counts[i]:] == -7), f"cell {i}: written past its row"
     assert np.all(np.abs(vol[cells] - ref["vol"]) <= 1e-5 * ref["vol"] + 1e-30)
+
+
+@pytest.mark.parametrize("n", [3_000, 60_000])
+@pytest.mark.parametrize("what", ["nan", "inf", "equal", "few"])
+def test_inputs_that_cull_nothing(vdmod, n, what):
+    """Sites without a finite position are reported, and copies of one position
+    leave one cell, without walks of the whole tree for each of them."""
+    x = W.uniform(n, 3)
+    if what in ("nan", "inf"):
+        x[::2] = np.nan if what == "nan" else np.inf
+        with pytest.raises(vdmod.VdError) as e:
+            vdmod.Context(0).build(torch.from_numpy(x).cuda(), None, W.UNIT_BOX)
+        assert e.value.code == vdmod.VD_ERR_INVALID_ARG
+        return
+    distinct = 1 if what == "equal" else 20
+    x = x[np.arange(n) % distinct]
+    res = vdmod.Context(0).build(torch.from_numpy(x).cuda(), None, W.UNIT_BOX)
+    vol = res.volume.double().cpu().numpy()
+    assert np.all(vol[distinct:] == 0) and abs(vol[:distinct].sum() - 1.0) <= 1e-5
+    if distinct > 1:
+        check(res, oracle.cells(x[:distinct]), np.arange(distinct))
