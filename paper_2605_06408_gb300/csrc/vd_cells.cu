@@ -1075,8 +1075,9 @@ bool uses_wide(const vd_config& g) { return g.cell_mode == 0 && !generic_config(
 
 // Four cells per warp from 192 sites per SM on (29,184 on GB300): a build of
 // fewer is bound by the latency of one warp's work, which is one cell here and
-// four there (and there a KNN query before it). By the sites of the whole
-// diagram, so that the parts of a partition agree with it to the last bit.
+// four there. Cells of uniform sites, one per warp and four: 10,000 sites 0.38
+// and 0.55 ms, 29,000 1.00 and 0.81 ms, 300,000 8.8 and 5.5 ms. By the sites of
+// the whole diagram, so that the parts of a partition agree with it to the last bit.
 bool uses_quad(const vd_config& g, int n, int num_sms) { return uses_wide(g) && n >= 192 * num_sms; }
 
 template <int VPL, int PCAP, int QPL>

@@ -22,7 +22,8 @@
 //   H  clip (all groups that found one).
 // Measured against one warp per cell (vd_cells.cu, as it was): 300,000
 // uniform sites 9.9 -> 5.2 ms, 1M in clusters 40.5 -> 24.4 ms, 2M on surfaces
-// 92 -> 58 ms; 13,000 warp instructions a cell instead of 22,000 to 29,000.
+// 92 -> 58 ms; warp instructions a cell 22,000 -> 12,700 (uniform) and
+// 29,000 -> 18,900 (surfaces).
 // Every collective runs on the whole warp and every loop ends on a warp vote
 // or a warp-uniform count (a group without work is masked).
 //
@@ -502,268 +503,268 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
 
 #pragma unroll 1
       while (true) {
-      // ---- F: candidates that leave every vertex inside are dropped for good
-      // (clipping only shrinks the cell); the nearest of the others is next
-      uint32_t key = 0xffffffffu;
-      {
-        int kept = 0;
+        // ---- F: candidates that leave every vertex inside are dropped for good
+        // (clipping only shrinks the cell); the nearest of the others is next
+        uint32_t key = 0xffffffffu;
+        {
+          int kept = 0;
 #pragma unroll 1
-        for (int base = 0; __any_sync(FULL, base < cn); base += 8) {
-          const int q = base + gl;
-          bool any = false;
-          float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
-          float he = 0.f;
-          int id = 0;
-          if (q < cn) {
-            h = S.cpl[q];
-            he = S.ce[q];
-            id = S.cid[q];
-            // the sign test's value plus both error bounds (a little more of
-            // each than the classification takes), as one chain per vertex
-            const float nb = fmaf(1.25f, he, -h.w);
-            float top = -INFINITY;
+          for (int base = 0; __any_sync(FULL, base < cn); base += 8) {
+            const int q = base + gl;
+            bool any = false;
+            float4 h = make_float4(0.f, 0.f, 0.f, 0.f);
+            float he = 0.f;
+            int id = 0;
+            if (q < cn) {
+              h = S.cpl[q];
+              he = S.ce[q];
+              id = S.cid[q];
+              // the sign test's value plus both error bounds (a little more of
+              // each than the classification takes), as one chain per vertex
+              const float nb = fmaf(1.25f, he, -h.w);
+              float top = -INFINITY;
 #pragma unroll 4
-            for (int v = 0; v < nv; v++) {
-              const float4 p = S.vp[v];
-              top = fmaxf(top, fmaf(h.x, p.x, fmaf(h.y, p.y, fmaf(h.z, p.z, fmaf(1.0001f, p.w, nb)))));
+              for (int v = 0; v < nv; v++) {
+                const float4 p = S.vp[v];
+                top = fmaxf(top, fmaf(h.x, p.x, fmaf(h.y, p.y, fmaf(h.z, p.z, fmaf(1.0001f, p.w, nb)))));
+              }
+              any = top > 0.f;
             }
-            any = top > 0.f;
+            __syncwarp();
+            const uint32_t km = group_ballot(any);
+            const int to = kept + __popc(km & ltg);
+            if (any) {
+              if (to != q) {
+                S.cpl[to] = h;
+                S.ce[to] = he;
+                S.cid[to] = id;
+              }
+              key = min(key, (f2o(h.w) & ~31u) | (uint32_t)to);
+            }
+            kept += __popc(km);
+            __syncwarp();
+          }
+          cn = kept;
+        }
+        const bool act = cn > 0;
+        if (!(clip_now ? __any_sync(FULL, act) : __any_sync(FULL, cn > kQS))) break;
+        clip_now = true;
+        // ---- C: classify the vertices
+        PlaneT<float> H;
+        H.nx = H.ny = H.nz = H.b = H.e = 0.f;
+        int hj = 0, k = 0;
+        uint32_t outm = 0;  // bit s: vertex 8 s + gl lies outside
+        bool cut = false;
+        {
+          key = group_minu(key);
+          if (act) {
+            const int at = (int)(key & 31u);
+            const float4 p = S.cpl[at];
+            H.nx = p.x;
+            H.ny = p.y;
+            H.nz = p.z;
+            H.b = p.w;
+            H.e = S.ce[at];
+            hj = S.cid[at];
           }
           __syncwarp();
-          const uint32_t km = group_ballot(any);
-          const int to = kept + __popc(km & ltg);
-          if (any) {
-            if (to != q) {
-              S.cpl[to] = h;
-              S.ce[to] = he;
-              S.cid[to] = id;
+          if (act) {  // the last candidate takes its place
+            const int at = (int)(key & 31u);
+            cn--;
+            if (gl == 0) {
+              S.cpl[at] = S.cpl[cn];
+              S.ce[at] = S.ce[cn];
+              S.cid[at] = S.cid[cn];
             }
-            key = min(key, (f2o(h.w) & ~31u) | (uint32_t)to);
           }
-          kept += __popc(km);
-          __syncwarp();
-        }
-        cn = kept;
-      }
-      const bool act = cn > 0;
-      if (!(clip_now ? __any_sync(FULL, act) : __any_sync(FULL, cn > kQS))) break;
-      clip_now = true;
-      // ---- C: classify the vertices
-      PlaneT<float> H;
-      H.nx = H.ny = H.nz = H.b = H.e = 0.f;
-      int hj = 0, k = 0;
-      uint32_t outm = 0;  // bit s: vertex 8 s + gl lies outside
-      bool cut = false;
-      {
-        key = group_minu(key);
-        if (act) {
-          const int at = (int)(key & 31u);
-          const float4 p = S.cpl[at];
-          H.nx = p.x;
-          H.ny = p.y;
-          H.nz = p.z;
-          H.b = p.w;
-          H.e = S.ce[at];
-          hj = S.cid[at];
-        }
-        __syncwarp();
-        if (act) {  // the last candidate takes its place
-          const int at = (int)(key & 31u);
-          cn--;
-          if (gl == 0) {
-            S.cpl[at] = S.cpl[cn];
-            S.ce[at] = S.ce[cn];
-            S.cid[at] = S.cid[cn];
-          }
-        }
-        uint32_t ambm = 0;
-        if (act) {
-          uint32_t bit = 1;
+          uint32_t ambm = 0;
+          if (act) {
+            uint32_t bit = 1;
 #pragma unroll 1
-          for (int v = gl; v < nv; v += 8, bit <<= 1) {
-            const float4 p = S.vp[v];
-            const float s = side<float>(H, p.x, p.y, p.z);
-            if (ambiguous<float>(s, p.w, H.e))
-              ambm |= bit;
-            else if (s > 0.0f)
-              outm |= bit;
-          }
-        }
-        __syncwarp();
-        if (__any_sync(FULL, ambm != 0)) {
-          while (ambm) {
-            const int s = __ffs(ambm) - 1;
-            ambm &= ambm - 1;
-            ct64++;
-            const unsigned r = walk_resolve64(S.pid, S.vt[8 * s + gl], hj, me, box, P.sites);
-            outm |= (r & 1u) << s;
-            ctamb += r >> 1;
+            for (int v = gl; v < nv; v += 8, bit <<= 1) {
+              const float4 p = S.vp[v];
+              const float s = side<float>(H, p.x, p.y, p.z);
+              if (ambiguous<float>(s, p.w, H.e))
+                ambm |= bit;
+              else if (s > 0.0f)
+                outm |= bit;
+            }
           }
           __syncwarp();
-        }
-        const int kk = group_add(__popc(outm));
-        if (act && kk > 0) {
-          k = kk;
-          if (k == nv) {
-            mode = M_EMPTY;
-            cn = 0;
-          } else {
-            cut = true;
+          if (__any_sync(FULL, ambm != 0)) {
+            while (ambm) {
+              const int s = __ffs(ambm) - 1;
+              ambm &= ambm - 1;
+              ct64++;
+              const unsigned r = walk_resolve64(S.pid, S.vt[8 * s + gl], hj, me, box, P.sites);
+              outm |= (r & 1u) << s;
+              ctamb += r >> 1;
+            }
+            __syncwarp();
           }
-        }
-      }
-
-      // ---- H: clip by the plane found (App. B)
-      if (!__any_sync(FULL, cut)) continue;
-      // a plane slot for it; slots that no kept vertex uses are reclaimed when none is free
-      if (__any_sync(FULL, cut && freem == 0)) {
-        uint32_t lo = 0, hi = 0;
-        if (cut) {
-          uint32_t bits = outm;
-          for (int v = gl; v < nv; v += 8, bits >>= 1) {
-            if (bits & 1u) continue;
-            const uint32_t T = S.vt[v];
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-              const uint32_t f = (T >> (8 * c)) & 255u;
-              if (f < 32u)
-                lo |= 1u << f;
-              else
-                hi |= 1u << (f - 32u);
+          const int kk = group_add(__popc(outm));
+          if (act && kk > 0) {
+            k = kk;
+            if (k == nv) {
+              mode = M_EMPTY;
+              cn = 0;
+            } else {
+              cut = true;
             }
           }
         }
+
+        // ---- H: clip by the plane found (App. B)
+        if (!__any_sync(FULL, cut)) continue;
+        // a plane slot for it; slots that no kept vertex uses are reclaimed when none is free
+        if (__any_sync(FULL, cut && freem == 0)) {
+          uint32_t lo = 0, hi = 0;
+          if (cut) {
+            uint32_t bits = outm;
+            for (int v = gl; v < nv; v += 8, bits >>= 1) {
+              if (bits & 1u) continue;
+              const uint32_t T = S.vt[v];
+#pragma unroll
+              for (int c = 0; c < 3; c++) {
+                const uint32_t f = (T >> (8 * c)) & 255u;
+                if (f < 32u)
+                  lo |= 1u << f;
+                else
+                  hi |= 1u << (f - 32u);
+              }
+            }
+          }
+          __syncwarp();
+          lo = group_or(lo);
+          hi = group_or(hi);
+          if (cut && freem == 0) freem = kQPlanes & ~(((uint64_t)hi << 32) | lo);
+          if (cut && freem == 0) {
+            mode = M_OVERFLOW;
+            cut = false;
+            cn = 0;
+          }
+        }
+        int h = 0;
+        if (cut) {
+          h = __ffsll((long long)freem) - 1;
+          freem &= freem - 1;
+          if (gl == 0) {
+            S.pl[h] = make_float4(H.nx, H.ny, H.nz, H.b);
+            S.pe[h] = H.e;
+            S.pid[h] = hj;
+          }
+        }
+        // the removed vertices' triplets and slots
+        int gone;
+        {
+          const int c = cut ? __popc(outm) : 0;
+          int before = c;
+#pragma unroll
+          for (int o = 1; o < 8; o <<= 1) {
+            const int t = __shfl_up_sync(FULL, before, o, 8);
+            if (gl >= o) before += t;
+          }
+          before -= c;
+          if (cut)
+            for (uint32_t bits = outm; bits; bits &= bits - 1) {
+              const int v = 8 * (__ffs(bits) - 1) + gl;
+              S.otri[before++] = S.vt[v] | ((uint32_t)v << 24);
+            }
+          gone = k;
+        }
         __syncwarp();
-        lo = group_or(lo);
-        hi = group_or(hi);
-        if (cut && freem == 0) freem = kQPlanes & ~(((uint64_t)hi << 32) | lo);
-        if (cut && freem == 0) {
+        // the hole's edges: every directed pair (a, b) of a removed vertex whose
+        // reverse is in no other removed vertex -> vertex (a, b, h). One removed
+        // vertex per lane
+        int m = 0;
+        {
+          const int kmax = __reduce_max_sync(FULL, cut ? k : 0);
+#pragma unroll 1
+          for (int base = 0; base < kmax; base += 8) {
+            const int t = base + gl;
+            const bool own = cut && t < k;
+            const uint32_t T = own ? S.otri[t] : 0u;
+            const uint32_t a = T & 255u, b = (T >> 8) & 255u, c = (T >> 16) & 255u;
+            const uint32_t r0 = b | (a << 8), r1 = c | (b << 8), r2 = a | (c << 8);
+            bool e0 = own, e1 = own, e2 = own;
+#pragma unroll 1
+            for (int v = 0; v < kmax; v++) {
+              const uint32_t U = v < k ? S.otri[v] : 0u;
+              const uint32_t p0 = U & 0xffffu, p1 = (U >> 8) & 0xffffu, p2 = ((U >> 16) & 255u) | ((U & 255u) << 8);
+              e0 = e0 && p0 != r0 && p1 != r0 && p2 != r0;
+              e1 = e1 && p0 != r1 && p1 != r1 && p2 != r1;
+              e2 = e2 && p0 != r2 && p1 != r2 && p2 != r2;
+            }
+            const uint32_t m0 = group_ballot(e0), m1 = group_ballot(e1), m2 = group_ballot(e2);
+            int at = m + __popc(m0 & ltg) + __popc(m1 & ltg) + __popc(m2 & ltg);
+            if (e0 && at < kQV) S.edge[at] = (unsigned short)(a | (b << 8));
+            at += e0;
+            if (e1 && at < kQV) S.edge[at] = (unsigned short)(b | (c << 8));
+            at += e1;
+            if (e2 && at < kQV) S.edge[at] = (unsigned short)(c | (a << 8));
+            m += __popc(m0) + __popc(m1) + __popc(m2);
+          }
+        }
+        if (cut && nv - gone + m > kQV) {
           mode = M_OVERFLOW;
           cut = false;
           cn = 0;
         }
-      }
-      int h = 0;
-      if (cut) {
-        h = __ffsll((long long)freem) - 1;
-        freem &= freem - 1;
-        if (gl == 0) {
-          S.pl[h] = make_float4(H.nx, H.ny, H.nz, H.b);
-          S.pe[h] = H.e;
-          S.pid[h] = hj;
-        }
-      }
-      // the removed vertices' triplets and slots
-      int gone;
-      {
-        const int c = cut ? __popc(outm) : 0;
-        int before = c;
-#pragma unroll
-        for (int o = 1; o < 8; o <<= 1) {
-          const int t = __shfl_up_sync(FULL, before, o, 8);
-          if (gl >= o) before += t;
-        }
-        before -= c;
-        if (cut)
-          for (uint32_t bits = outm; bits; bits &= bits - 1) {
-            const int v = 8 * (__ffs(bits) - 1) + gl;
-            S.otri[before++] = S.vt[v] | ((uint32_t)v << 24);
-          }
-        gone = k;
-      }
-      __syncwarp();
-      // the hole's edges: every directed pair (a, b) of a removed vertex whose
-      // reverse is in no other removed vertex -> vertex (a, b, h). One removed
-      // vertex per lane
-      int m = 0;
-      {
-        const int kmax = __reduce_max_sync(FULL, cut ? k : 0);
+        __syncwarp();
+        // new vertex t takes the slot of removed vertex t, then slots at the end
 #pragma unroll 1
-        for (int base = 0; base < kmax; base += 8) {
+        for (int base = 0; __any_sync(FULL, cut && base < m); base += 8) {
           const int t = base + gl;
-          const bool own = cut && t < k;
-          const uint32_t T = own ? S.otri[t] : 0u;
-          const uint32_t a = T & 255u, b = (T >> 8) & 255u, c = (T >> 16) & 255u;
-          const uint32_t r0 = b | (a << 8), r1 = c | (b << 8), r2 = a | (c << 8);
-          bool e0 = own, e1 = own, e2 = own;
-#pragma unroll 1
-          for (int v = 0; v < kmax; v++) {
-            const uint32_t U = v < k ? S.otri[v] : 0u;
-            const uint32_t p0 = U & 0xffffu, p1 = (U >> 8) & 0xffffu, p2 = ((U >> 16) & 255u) | ((U & 255u) << 8);
-            e0 = e0 && p0 != r0 && p1 != r0 && p2 != r0;
-            e1 = e1 && p0 != r1 && p1 != r1 && p2 != r1;
-            e2 = e2 && p0 != r2 && p1 != r2 && p2 != r2;
-          }
-          const uint32_t m0 = group_ballot(e0), m1 = group_ballot(e1), m2 = group_ballot(e2);
-          int at = m + __popc(m0 & ltg) + __popc(m1 & ltg) + __popc(m2 & ltg);
-          if (e0 && at < kQV) S.edge[at] = (unsigned short)(a | (b << 8));
-          at += e0;
-          if (e1 && at < kQV) S.edge[at] = (unsigned short)(b | (c << 8));
-          at += e1;
-          if (e2 && at < kQV) S.edge[at] = (unsigned short)(c | (a << 8));
-          m += __popc(m0) + __popc(m1) + __popc(m2);
-        }
-      }
-      if (cut && nv - gone + m > kQV) {
-        mode = M_OVERFLOW;
-        cut = false;
-        cn = 0;
-      }
-      __syncwarp();
-      // new vertex t takes the slot of removed vertex t, then slots at the end
-#pragma unroll 1
-      for (int base = 0; __any_sync(FULL, cut && base < m); base += 8) {
-        const int t = base + gl;
-        if (cut && t < m) {
-          const uint32_t ab = S.edge[t];
-          const int a = (int)(ab & 255u), b = (int)(ab >> 8);
-          const int at = t < gone ? (int)(S.otri[t] >> 24) : nv + (t - gone);
-          float x, y, z, ev;
-          vertex3<float>(quad_plane(S, a), quad_plane(S, b), H, x, y, z, ev);
-          S.vp[at] = make_float4(x, y, z, ev);
-          S.vt[at] = ab | ((uint32_t)h << 16);
-          if (!(ev <= kRefineRel * (fabsf(x) + fabsf(y) + fabsf(z)))) {
-            walk_refine(&S.vp[at], S.pid[a], S.pid[b], hj, me, box, P.sites);
-            ctrefv++;
+          if (cut && t < m) {
+            const uint32_t ab = S.edge[t];
+            const int a = (int)(ab & 255u), b = (int)(ab >> 8);
+            const int at = t < gone ? (int)(S.otri[t] >> 24) : nv + (t - gone);
+            float x, y, z, ev;
+            vertex3<float>(quad_plane(S, a), quad_plane(S, b), H, x, y, z, ev);
+            S.vp[at] = make_float4(x, y, z, ev);
+            S.vt[at] = ab | ((uint32_t)h << 16);
+            if (!(ev <= kRefineRel * (fabsf(x) + fabsf(y) + fabsf(z)))) {
+              walk_refine(&S.vp[at], S.pid[a], S.pid[b], hj, me, box, P.sites);
+              ctrefv++;
+            }
           }
         }
-      }
-      __syncwarp();
-      // fewer new vertices than removed ones: the slots left over are filled
-      // from the end of the array
-      if (__any_sync(FULL, cut && m < gone)) {
-        const int left = cut ? max(gone - m, 0) : 0, to = nv - left;
-        for (int t = gl; t < left; t += 8) S.vt[S.otri[m + t] >> 24] = kEmptyTri;
         __syncwarp();
-        int holes = 0, live = 0;
-        const int lmax = __reduce_max_sync(FULL, left);
+        // fewer new vertices than removed ones: the slots left over are filled
+        // from the end of the array
+        if (__any_sync(FULL, cut && m < gone)) {
+          const int left = cut ? max(gone - m, 0) : 0, to = nv - left;
+          for (int t = gl; t < left; t += 8) S.vt[S.otri[m + t] >> 24] = kEmptyTri;
+          __syncwarp();
+          int holes = 0, live = 0;
+          const int lmax = __reduce_max_sync(FULL, left);
 #pragma unroll 1
-        for (int base = 0; base < lmax; base += 8) {
-          const int t = base + gl;
-          const int slot = t < left ? (int)(S.otri[m + t] >> 24) : kQV;
-          const uint32_t hm = group_ballot(slot < to);
-          if (slot < to) S.edge[holes + __popc(hm & ltg)] = (unsigned short)slot;
-          holes += __popc(hm);
-        }
-        __syncwarp();
-#pragma unroll 1
-        for (int base = 0; base < lmax; base += 8) {
-          const int v = to + base + gl;
-          const bool mv = base + gl < left && S.vt[v] != kEmptyTri;
-          const uint32_t vm = group_ballot(mv);
-          if (mv) {
-            const int slot = (int)S.edge[live + __popc(vm & ltg)];
-            S.vp[slot] = S.vp[v];
-            S.vt[slot] = S.vt[v];
+          for (int base = 0; base < lmax; base += 8) {
+            const int t = base + gl;
+            const int slot = t < left ? (int)(S.otri[m + t] >> 24) : kQV;
+            const uint32_t hm = group_ballot(slot < to);
+            if (slot < to) S.edge[holes + __popc(hm & ltg)] = (unsigned short)slot;
+            holes += __popc(hm);
           }
-          live += __popc(vm);
+          __syncwarp();
+#pragma unroll 1
+          for (int base = 0; base < lmax; base += 8) {
+            const int v = to + base + gl;
+            const bool mv = base + gl < left && S.vt[v] != kEmptyTri;
+            const uint32_t vm = group_ballot(mv);
+            if (mv) {
+              const int slot = (int)S.edge[live + __popc(vm & ltg)];
+              S.vp[slot] = S.vp[v];
+              S.vt[slot] = S.vt[v];
+            }
+            live += __popc(vm);
+          }
+          __syncwarp();
         }
-        __syncwarp();
-      }
-      if (cut) {
-        nv += m - gone;
-        dirty = true;
-      }
+        if (cut) {
+          nv += m - gone;
+          dirty = true;
+        }
       }
       cf = cn;
       if (finished || !__any_sync(FULL, mode == M_BUILD)) break;

@@ -51,7 +51,10 @@ enum { S_BUILD = 0, S_EMPTY = 1, S_FULL = 2, S_FAR = 3, S_PLANES = 4, S_ROW = 5 
 
 // Volume and first moment about (cx, cy, cz) in FP64 (the scheme of
 // volume_fp64). Overwrites vp, pl and pe.
-__device__ __noinline__ double4 solo_volume64(SoloCell& S, int nv, float4 me, const float* box,
+struct SoloMoments {
+  double v, x, y, z;
+};
+__device__ __noinline__ SoloMoments solo_volume64(SoloCell& S, int nv, float4 me, const float* box,
                                               const float4* __restrict__ sites, double cx, double cy, double cz) {
   const int lane = (int)lane_id();
   double* vd64 = reinterpret_cast<double*>(S.vp);
@@ -100,7 +103,7 @@ __device__ __noinline__ double4 solo_volume64(SoloCell& S, int nv, float4 me, co
     My += __shfl_xor_sync(FULL, My, o);
     Mz += __shfl_xor_sync(FULL, Mz, o);
   }
-  return make_double4(V / 6.0, Mx / 24.0, My / 24.0, Mz / 24.0);
+  return SoloMoments{V / 6.0, Mx / 24.0, My / 24.0, Mz / 24.0};
 }
 
 // A plane slot that no vertex uses but the k about to be removed (otri), or
@@ -460,81 +463,81 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           }
           steps += 64;
         } else {
-        if (pend == 0) {
-          if (qn == 0 && cur < 0) {
-            finished = true;
-            break;
-          }
-          steps++;
-          uint32_t todo = 255u;
-          int ref = lane < 8 ? cur : -1;
-          if (cur < 0) ref = solo_pop(S, qn, todo);
-          cur = -1;
-          bool keep = false;
-          float key = 0.f;
-          if (ref >= 0) {
-            const float4* nd = P.wide + 16 * (size_t)ref + (lane & 7);
-            const float4 lo = __ldg(nd), hi = __ldg(nd + 8);
-            cref = __float_as_int(hi.w);
-            float lb;
-            keep = walk_node_test(lo, hi, me, B, weighted, key, lb) && cref != kNoChild && ((todo >> (lane & 7)) & 1u);
-            // a long walk: test the cone of directions toward the box too (see
-            // node_cone), against the cell's exact support in the cone's axis
-            if (steps > kSCone && keep) keep = solo_cone_test(S.vp, nv, lo, hi, me, lb, B.reach2);
-          } else {  // none, or a set of one leaf
-            cref = SI.wroot;
-            keep = lane == 0 && ref_is_leaf(cref);
-          }
-          pend = __ballot_sync(FULL, keep && ref_is_leaf(cref));
-          const bool inner = keep && !ref_is_leaf(cref);
-          const uint32_t im = __ballot_sync(FULL, inner);
-          if (im && qn + __popc(im) > kSQ - 24) {
-            // little room (bounds still loose in several directions; one node
-            // was visited): go on with the best child, and queue the node
-            // itself with the others, to be tested again under the bounds of
-            // that time
-            const uint32_t kk = inner ? f2o(key) & ~0x7fffu : 0xffffffffu;
-            const uint32_t b1 = __reduce_min_sync(FULL, inner ? (kk | (uint32_t)lane) : 0xffffffffu);
-            const int src = (int)(b1 & 31u);
-            const uint32_t rest = im & ~(1u << src);
-            cur = __shfl_sync(FULL, cref, src);
-            if (rest) {
-              if (qn >= kSQ || im > 255u) {
-                mode = S_FAR;
-                break;
-              }
-              const uint32_t b2 = __reduce_min_sync(FULL, lane != src ? kk : 0xffffffffu);
-              if (lane == 0) {
-                S.q[qn] = (b2 & ~0x7fffu) | (rest << 7);
-                S.q[kSQ + qn] = ref;
-              }
-              qn++;
+          if (pend == 0) {
+            if (qn == 0 && cur < 0) {
+              finished = true;
+              break;
             }
+            steps++;
+            uint32_t todo = 255u;
+            int ref = lane < 8 ? cur : -1;
+            if (cur < 0) ref = solo_pop(S, qn, todo);
+            cur = -1;
+            bool keep = false;
+            float key = 0.f;
+            if (ref >= 0) {
+              const float4* nd = P.wide + 16 * (size_t)ref + (lane & 7);
+              const float4 lo = __ldg(nd), hi = __ldg(nd + 8);
+              cref = __float_as_int(hi.w);
+              float lb;
+              keep = walk_node_test(lo, hi, me, B, weighted, key, lb) && cref != kNoChild && ((todo >> (lane & 7)) & 1u);
+              // a long walk: test the cone of directions toward the box too (see
+              // node_cone), against the cell's exact support in the cone's axis
+              if (steps > kSCone && keep) keep = solo_cone_test(S.vp, nv, lo, hi, me, lb, B.reach2);
+            } else {  // none, or a set of one leaf
+              cref = SI.wroot;
+              keep = lane == 0 && ref_is_leaf(cref);
+            }
+            pend = __ballot_sync(FULL, keep && ref_is_leaf(cref));
+            const bool inner = keep && !ref_is_leaf(cref);
+            const uint32_t im = __ballot_sync(FULL, inner);
+            if (im && qn + __popc(im) > kSQ - 24) {
+              // little room (bounds still loose in several directions; one node
+              // was visited): go on with the best child, and queue the node
+              // itself with the others, to be tested again under the bounds of
+              // that time
+              const uint32_t kk = inner ? f2o(key) & ~0x7fffu : 0xffffffffu;
+              const uint32_t b1 = __reduce_min_sync(FULL, inner ? (kk | (uint32_t)lane) : 0xffffffffu);
+              const int src = (int)(b1 & 31u);
+              const uint32_t rest = im & ~(1u << src);
+              cur = __shfl_sync(FULL, cref, src);
+              if (rest) {
+                if (qn >= kSQ || im > 255u) {
+                  mode = S_FAR;
+                  break;
+                }
+                const uint32_t b2 = __reduce_min_sync(FULL, lane != src ? kk : 0xffffffffu);
+                if (lane == 0) {
+                  S.q[qn] = (b2 & ~0x7fffu) | (rest << 7);
+                  S.q[kSQ + qn] = ref;
+                }
+                qn++;
+              }
+              __syncwarp();
+              continue;
+            }
+            if (inner) {
+              const int to = qn + __popc(im & lt);
+              S.q[to] = (f2o(key) & ~0x7fffu) | (255u << 7);
+              S.q[kSQ + to] = cref;
+            }
+            qn += __popc(im);
             __syncwarp();
             continue;
           }
-          if (inner) {
-            const int to = qn + __popc(im & lt);
-            S.q[to] = (f2o(key) & ~0x7fffu) | (255u << 7);
-            S.q[kSQ + to] = cref;
-          }
-          qn += __popc(im);
-          __syncwarp();
-          continue;
-        }
-        // read up to four leaves, two at a time
+          // read up to four leaves, two at a time
 #pragma unroll
-        for (int r = 0; r < 2; r++) {
-          const int c0 = __ffs(pend) - 1;
-          const uint32_t p1 = pend & (pend - 1);
-          const int c1 = __ffs(p1) - 1;
-          pend = p1 & (p1 - 1);
-          const int c = lane < 16 ? c0 : c1;
-          const int ref = __shfl_sync(FULL, cref, c & 31);
-          j[r] = leaf_first(ref) + (lane & 15);
-          act[r] = (c >= 0) & ((lane & 15) < leaf_count(ref)) & (j[r] != si) & ((j[r] < w0) | (j[r] >= w1));
-          q[r] = P.sites[act[r] ? j[r] : si];
-        }
+          for (int r = 0; r < 2; r++) {
+            const int c0 = __ffs(pend) - 1;
+            const uint32_t p1 = pend & (pend - 1);
+            const int c1 = __ffs(p1) - 1;
+            pend = p1 & (p1 - 1);
+            const int c = lane < 16 ? c0 : c1;
+            const int ref = __shfl_sync(FULL, cref, c & 31);
+            j[r] = leaf_first(ref) + (lane & 15);
+            act[r] = (c >= 0) & ((lane & 15) < leaf_count(ref)) & (j[r] != si) & ((j[r] < w0) | (j[r] >= w1));
+            q[r] = P.sites[act[r] ? j[r] : si];
+          }
         }
         bool dup = false;
 #pragma unroll
@@ -890,13 +893,13 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
         L = sqrtf(L);
         double ox = cx, oy = cy, oz = cz, Vd = V;
         if (volume_needs_fp64(V, L, Sabs, emax)) {
-          const double4 r = solo_volume64(S, nv, me, box, P.sites, (double)cx, (double)cy, (double)cz);
-          Vd = r.x;
+          const SoloMoments r = solo_volume64(S, nv, me, box, P.sites, (double)cx, (double)cy, (double)cz);
+          Vd = r.v;
           if (Vd > 0.0) {
             const double iv = 1.0 / Vd;
-            ox += r.y * iv;
-            oy += r.z * iv;
-            oz += r.w * iv;
+            ox += r.x * iv;
+            oy += r.y * iv;
+            oz += r.z * iv;
           }
           if (lane == 0) ctrefvol++;
         } else if (V > 0.0f) {
@@ -931,7 +934,10 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
       set_error(P.st, VD_ERR_CELL_OVERFLOW);
     }
     if (!BRUTE && mode > S_EMPTY && lane == 0) {  // to the large-cell pass
-      const int reason = mode == S_FULL ? OVF_VERTICES : mode == S_FAR ? OVF_QUEUE : mode == S_PLANES ? OVF_PLANES : OVF_NEIGHBORS;
+      const int reason = mode == S_FULL     ? OVF_VERTICES
+                         : mode == S_FAR    ? OVF_QUEUE
+                         : mode == S_PLANES ? OVF_PLANES
+                                            : OVF_NEIGHBORS;
       ctovf++;
       atomicAdd((unsigned long long*)&P.st->ovf_reason[reason], 1ull);
       P.ovf_list[atomicAdd(&P.st->ovf_count, 1)] = si;
