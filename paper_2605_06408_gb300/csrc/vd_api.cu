@@ -393,7 +393,7 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   ctx->perm = v0;
   mark(ctx, 2, s);
   // 3. packed float4 sites in Morton order (App. A.1)
-  e = launch_gather_sites(xyz, w, ctx->perm, n, ctx->sets_dev, ctx->keys_sorted, set_shift, nsets, ctx->sites,
+  e = launch_gather_sites(xyz, w, ctx->perm, n, ctx->sets_dev, ctx->keys_sorted, set_shift, nsets, ctx->st, ctx->sites,
                           ctx->inv_perm, ctx->loser, s);
   if (e != cudaSuccess) return VD_ERR_CUDA;
   // 4. LBVH with per-node max weight (App. A.2)

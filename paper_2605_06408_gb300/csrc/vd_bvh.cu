@@ -24,7 +24,7 @@ __device__ __forceinline__ uint64_t spread3(uint32_t v) {
   return x;
 }
 
-__device__ __forceinline__ int find_set(const SetInfo* sets, int nsets, int i) {
+__host__ __device__ __forceinline__ int find_set(const SetInfo* sets, int nsets, int i) {
   int lo = 0, hi = nsets - 1;
   while (lo < hi) {
     int mid = (lo + hi + 1) >> 1;
@@ -148,8 +148,10 @@ cudaError_t launch_pack_keys(const float* xyz, const float* w, int n, const SetI
 // time of the passes' bytes at the copy rate).
 //
 // Tiles are numbered in the order in which their blocks start, so a tile only
-// waits for tiles that are running or done; the wait is bounded all the same
-// (VD_ERR_TIMEOUT; positions are clamped to the array).
+// waits for tiles that are running or done; the wait is bounded all the same.
+// A tile whose wait runs out writes nothing: it reports VD_ERR_TIMEOUT and sets
+// sort_failed, at which every later tile and pass stops (the arrays hold no
+// permutation any more) and gather_sites_kernel starts from the input's order.
 
 constexpr int kSortThreads = 256;
 constexpr int kSortWarps = kSortThreads / 32;
@@ -173,10 +175,15 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_kernel(const uint64_t*
   __shared__ int sv[TILE];
   __shared__ int tile_id;
   const int t = (int)threadIdx.x, lane = t & 31, w = t >> 5;
-  if (t == 0) tile_id = (int)atomicAdd(ticket, 1u);
+  if (t == 0) {
+    const int failed = *(volatile const int*)&st->sort_failed;
+    const int id = (int)atomicAdd(ticket, 1u);
+    tile_id = failed ? -1 : id;
+  }
   for (int k = t; k < kSortWarps * 256; k += kSortThreads) (&wh[0][0])[k] = 0;
   __syncthreads();
   const int tile = tile_id;
+  if (tile < 0) return;
   next_chain[(size_t)tile * 256 + t] = 0;  // the next pass's chain, idle during this one
   const int base = tile * TILE + w * 32 * ITEMS + lane;
   uint64_t key[ITEMS];
@@ -233,13 +240,15 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_kernel(const uint64_t*
 #pragma unroll
   for (int q = 0; q < kSortWarps; q++) wh[q][t] += a;
   unsigned sum = 0;
+  bool lost = false;
   if (tile > 0) {
     int waits = 0;
     for (int p = tile - 1; p >= 0;) {
       const unsigned v = chain[(size_t)p * 256 + t];
       if (v < kSortOwn) {
-        if (++waits > kSortWaitLimit) {
-          set_error(st, VD_ERR_TIMEOUT);
+        // a tile that stopped publishes nothing: look for the mark now and then
+        if (++waits > kSortWaitLimit || ((waits & 1023) == 0 && *(volatile const int*)&st->sort_failed)) {
+          lost = true;
           break;
         }
         continue;
@@ -248,10 +257,16 @@ __global__ void __launch_bounds__(kSortThreads) sort_pass_kernel(const uint64_t*
       if (v >= kSortSum) break;
       p--;
     }
-    chain[(size_t)tile * 256 + t] = (count + sum) | kSortSum;
+    if (!lost) chain[(size_t)tile * 256 + t] = (count + sum) | kSortSum;
   }
   place[t] = (int)(b + sum) - (int)a;
-  __syncthreads();
+  if (__syncthreads_or(lost)) {
+    if (t == 0) {
+      set_error(st, VD_ERR_TIMEOUT);
+      atomicExch(&st->sort_failed, 1);
+    }
+    return;
+  }
 #pragma unroll
   for (int i = 0; i < ITEMS; i++) {
     const int at = base + 32 * i;
@@ -410,38 +425,53 @@ cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, i
 // larger weight, then the lower original index, keeps its cell; every other
 // one has an empty cell, and its half-space is implied by the winner's, so it
 // is never a candidate.
-__global__ void gather_sites_kernel(const float* __restrict__ xyz, const float* __restrict__ w,
-                                    const int* __restrict__ perm, int n, const SetInfo* __restrict__ sets,
-                                    const uint64_t* __restrict__ keys, int set_shift, int nsets,
-                                    float4* __restrict__ sites, int* __restrict__ inv,
-                                    unsigned char* __restrict__ loser) {
-  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x) {
-    const int i = perm[k];
-    const uint64_t key = keys[k];
-    const int s = nsets > 1 ? (int)(key >> set_shift) : 0;
-    const bool weighted = w && sets[s].weighted;
-    const float4 p = make_float4(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], weighted ? w[i] : 0.0f);
-    sites[k] = p;
-    inv[i] = k;
-    bool lose = false;
-    for (int dir = -1; dir <= 1 && !lose; dir += 2)
-      for (int m = k + dir; m >= 0 && m < n && keys[m] == key && !lose; m += dir) {
-        const int o = perm[m];
-        if (xyz[3 * o] == p.x && xyz[3 * o + 1] == p.y && xyz[3 * o + 2] == p.z) {
-          const float qw = weighted ? w[o] : 0.0f;
-          lose = qw > p.w || (qw == p.w && o < i);
-        }
-      }
-    loser[k] = lose ? 1 : 0;
+//
+// After a sort that gave up (`failed`), perm and keys hold whatever was in the
+// arrays: every place takes the input's own order instead, with keys of the
+// set alone (sorted, so the tree over them is a valid one), and every site is a
+// loser, so that no cell is made of it: the build ends with empty rows and
+// VD_ERR_TIMEOUT. One place, for the host too (that order is tested there).
+__host__ __device__ inline void gather_site(const float* xyz, const float* w, int* perm, int n, const SetInfo* sets,
+                                            uint64_t* keys, int set_shift, int nsets, bool failed, float4* sites,
+                                            int* inv, unsigned char* loser, int k) {
+  if (failed) {
+    perm[k] = k;
+    keys[k] = nsets > 1 ? (uint64_t)find_set(sets, nsets, k) << set_shift : 0;
   }
+  const int i = perm[k];
+  const uint64_t key = keys[k];
+  const int s = nsets > 1 ? (int)(key >> set_shift) : 0;
+  const bool weighted = w && sets[s].weighted;
+  const float4 p = make_float4(xyz[3 * i], xyz[3 * i + 1], xyz[3 * i + 2], weighted ? w[i] : 0.0f);
+  sites[k] = p;
+  inv[i] = k;
+  bool lose = failed;
+  for (int dir = -1; dir <= 1 && !lose; dir += 2)
+    for (int m = k + dir; m >= 0 && m < n && keys[m] == key && !lose; m += dir) {
+      const int o = perm[m];
+      if (xyz[3 * o] == p.x && xyz[3 * o + 1] == p.y && xyz[3 * o + 2] == p.z) {
+        const float qw = weighted ? w[o] : 0.0f;
+        lose = qw > p.w || (qw == p.w && o < i);
+      }
+    }
+  loser[k] = lose ? 1 : 0;
 }
 
-cudaError_t launch_gather_sites(const float* xyz, const float* w, const int* perm, int n, const SetInfo* sets,
-                                const uint64_t* keys, int set_shift, int nsets, float4* sites, int* inv,
+__global__ void gather_sites_kernel(const float* __restrict__ xyz, const float* __restrict__ w, int* __restrict__ perm,
+                                    int n, const SetInfo* __restrict__ sets, uint64_t* __restrict__ keys, int set_shift,
+                                    int nsets, const DevStatus* __restrict__ st, float4* __restrict__ sites,
+                                    int* __restrict__ inv, unsigned char* __restrict__ loser) {
+  const bool failed = st->sort_failed != 0;
+  for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < n; k += gridDim.x * blockDim.x)
+    gather_site(xyz, w, perm, n, sets, keys, set_shift, nsets, failed, sites, inv, loser, k);
+}
+
+cudaError_t launch_gather_sites(const float* xyz, const float* w, int* perm, int n, const SetInfo* sets, uint64_t* keys,
+                                int set_shift, int nsets, const DevStatus* st, float4* sites, int* inv,
                                 unsigned char* loser, cudaStream_t s) {
   int threads = 256;
   int blocks = min((n + threads - 1) / threads, 4096);
-  gather_sites_kernel<<<blocks, threads, 0, s>>>(xyz, w, perm, n, sets, keys, set_shift, nsets, sites, inv, loser);
+  gather_sites_kernel<<<blocks, threads, 0, s>>>(xyz, w, perm, n, sets, keys, set_shift, nsets, st, sites, inv, loser);
   return cudaGetLastError();
 }
 

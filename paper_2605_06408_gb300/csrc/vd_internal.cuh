@@ -71,6 +71,8 @@ struct DevStatus {
   long long btape_restored;  // ... restored from it by the last adjoint
   int amb_count;             // cells with an FP64 sign test left inside its bound
   int mid_count;             // cells the four-per-warp kernel left to the one-per-warp kernel
+  int sort_failed;           // a tile of the sort gave up waiting (VD_ERR_TIMEOUT)
+  int pad;
 };
 
 // Record cell `orig` (original index) as one whose construction took an FP64
@@ -358,8 +360,8 @@ size_t sort_scratch_bytes(int64_t n);
 size_t sort_clear_words(int n);
 cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, int*& vals_alt, unsigned* scratch, int n,
                              int bits, DevStatus* st, cudaStream_t s);
-cudaError_t launch_gather_sites(const float* xyz, const float* w, const int* perm, int n, const SetInfo* sets,
-                                const uint64_t* keys, int set_shift, int nsets, float4* sites, int* inv,
+cudaError_t launch_gather_sites(const float* xyz, const float* w, int* perm, int n, const SetInfo* sets, uint64_t* keys,
+                                int set_shift, int nsets, const DevStatus* st, float4* sites, int* inv,
                                 unsigned char* loser, cudaStream_t s);
 cudaError_t launch_build_bvh(const uint64_t* keys, const float4* sites, int n, int leaf_size, BvhBuffers& b,
                              SetInfo* sets, int nsets, DevStatus* st, cudaStream_t s);
