@@ -653,6 +653,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
             if (out) S.otri[k + __popc(om & lt)] = S.vt[v] | ((uint32_t)v << 24);
             k += __popc(om);
           }
+          __syncwarp();  // the list: read by other lanes in solo_reclaim already
           if (k == 0) continue;
           if (k == nv) {
             mode = S_EMPTY;
@@ -737,6 +738,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           dirty = true;
         }
       }
+      __syncwarp();  // the candidates have been read: the walk puts others in their places
       cn = 0;
       first = false;
       if (finished) break;
