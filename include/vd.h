@@ -299,8 +299,9 @@ int vd_get_status(vd_ctx* ctx, vd_status* st);
  * cells against exact arithmetic (a project addition: the paper runs FP32
  * only and reports no such set). Synchronises the context's last stream.
  *   cells    : HOST int64 [capacity]: original site indices (global indices
- *              for batched builds), in no particular order; a cell re-run by
- *              the large-cell pass may appear twice.
+ *              for batched builds), in no particular order; each once in the
+ *              default modes (in the others a cell re-run by the large-cell
+ *              pass may appear twice).
  *   capacity : entries `cells` holds (0 with cells = NULL: count only).
  *   count    : HOST scalar: how many were recorded; at most the first 65,536
  *              are kept, so count > 65,536 means the list is truncated.

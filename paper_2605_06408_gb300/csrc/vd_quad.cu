@@ -63,7 +63,8 @@ struct __align__(16) QuadCell {
   float ce[kQC];
   int cid[kQC];
   int knn[kKnn];
-  int pad[8];
+  unsigned tally[8];  // of the group's finished cells: FP64 signs, those still ambiguous, vertices and volumes re-solved,
+                      // empty cells
 };
 static_assert(sizeof(QuadCell) % 128 == 32, "bank layout");
 struct __align__(16) QuadWarp {
@@ -75,6 +76,7 @@ static_assert(kQF * kQF <= kQC * (16 + 4 + 4), "edge table over the candidate ar
 static_assert(kKnn == 8, "one KNN site per lane of a group");
 static_assert(sizeof(double) * 3 * kQV <= sizeof(float4) * (kQV + kQP), "FP64 scratch");
 
+enum { T_SIGNS = 0, T_AMB = 1, T_VERTS = 2, T_VOLS = 3, T_EMPTY = 4, T_COUNT = 5 };
 enum { M_BUILD = 0, M_EMPTY = 1, M_OVERFLOW = 2, M_IDLE = 3 };
 
 // reductions over the 8 lanes of a group
@@ -208,8 +210,8 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
   QuadWarp& W = reinterpret_cast<QuadWarp*>(quad_smem)[threadIdx.x >> 5];
   QuadCell& S = W.cell[lane >> 3];
   auto group_ballot = [&](bool p) { return (__ballot_sync(FULL, p) >> gsh) & 255u; };
-  unsigned ct64 = 0, ctamb = 0, ctrefv = 0, ctrefvol = 0, ctempty = 0;
   const float u = Num<float>::u;
+  S.tally[gl] = 0;
 
   while (true) {
     int item = 0;
@@ -228,7 +230,7 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
     const float* box = SI.lo;
     // a site that an exact duplicate beats has an empty cell
     int mode = !exists ? M_IDLE : (P.loser[si] || !finite_site(me) ? M_EMPTY : M_BUILD);
-    const unsigned amb0 = ctamb;
+    unsigned ct64 = 0, ctamb = 0, ctrefv = 0;  // this cell's, a lane's share
 
     // ---- the box: 6 planes, 8 corners (as init_cell)
     if (gl < 6) {
@@ -774,7 +776,7 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
     if (!own) mode = M_IDLE;
     if (mode == M_EMPTY) {
       if (gl == 0) {
-        ctempty++;
+        S.tally[T_EMPTY]++;
         P.counts[orig] = 0;
         P.vol[orig] = 0.0f;
         P.cen[3 * (size_t)orig] = me.x;
@@ -914,7 +916,7 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
             oy += Y6 * iv;
             oz += Z6 * iv;
           }
-          if (gl == 0) ctrefvol++;
+          if (gl == 0) S.tally[T_VOLS]++;
         }
       }
       if (!need64 && V > 0.0f) {
@@ -930,21 +932,32 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
         P.cen[3 * (size_t)orig + 2] = (float)((double)me.z + oz);
       }
     }
-    const uint32_t am = group_ballot(ctamb != amb0);
-    if (own && am && gl == 0) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+    // the events of cells that this kernel finishes: of one passed on, the next
+    // kernel counts them, of a neighbouring part's cell, that part's build
+    const bool kept = mode == M_BUILD || mode == M_EMPTY;
+    if (__any_sync(FULL, kept && (ct64 | ctrefv) != 0)) {
+      const unsigned signs = (unsigned)group_add((int)ct64), amb = (unsigned)group_add((int)ctamb),
+                     verts = (unsigned)group_add((int)ctrefv);
+      if (kept && gl == 0) {
+        S.tally[T_SIGNS] += signs;
+        S.tally[T_AMB] += amb;
+        S.tally[T_VERTS] += verts;
+        if (amb) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+      }
+    }
     __syncwarp();
   }
-  ct64 = __reduce_add_sync(FULL, ct64);
-  ctamb = __reduce_add_sync(FULL, ctamb);
-  ctrefv = __reduce_add_sync(FULL, ctrefv);
-  ctrefvol = __reduce_add_sync(FULL, ctrefvol);
-  ctempty = __reduce_add_sync(FULL, ctempty);
-  if (lane == 0) {
-    if (ct64) atomicAdd((unsigned long long*)&P.st->fp64_fallbacks, (unsigned long long)ct64);
-    if (ctamb) atomicAdd((unsigned long long*)&P.st->fp64_ambiguous, (unsigned long long)ctamb);
-    if (ctrefv) atomicAdd((unsigned long long*)&P.st->refined_vertices, (unsigned long long)ctrefv);
-    if (ctrefvol) atomicAdd((unsigned long long*)&P.st->refined_volumes, (unsigned long long)ctrefvol);
-    if (ctempty) atomicAdd((unsigned long long*)&P.st->empty_cells, (unsigned long long)ctempty);
+  __syncwarp();
+  unsigned sum = S.tally[gl];
+  sum += __shfl_xor_sync(FULL, sum, 8);
+  sum += __shfl_xor_sync(FULL, sum, 16);
+  if (lane < T_COUNT && sum) {
+    long long* to = lane == T_SIGNS   ? &P.st->fp64_fallbacks
+                    : lane == T_AMB   ? &P.st->fp64_ambiguous
+                    : lane == T_VERTS ? &P.st->refined_vertices
+                    : lane == T_VOLS  ? &P.st->refined_volumes
+                                      : &P.st->empty_cells;
+    atomicAdd((unsigned long long*)to, (unsigned long long)sum);
   }
 }
 

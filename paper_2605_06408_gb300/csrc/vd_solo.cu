@@ -43,6 +43,7 @@ struct __align__(16) SoloCell {
                         // at the end the neighbour list
   unsigned char fill[kSV];  // slots to fill
   uint32_t freep[kSP / 32];  // plane slots reclaimed once all have been used
+  unsigned tally[4];  // of the warp's finished cells: FP64 signs, those still ambiguous, vertices re-solved
 };
 static_assert(kSF * kSF <= kSC * 16, "edge table over the candidates");
 static_assert(sizeof(double) * 3 * kSV <= sizeof(float4) * (kSV + kSP), "FP64 scratch");
@@ -312,7 +313,8 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
   const int lane = (int)lane_id();
   const uint32_t lt = lanemask_lt();
   const float u = Num<float>::u;
-  unsigned ct64 = 0, ctamb = 0, ctrefv = 0, ctrefvol = 0, ctempty = 0, ctovf = 0;
+  unsigned ctrefvol = 0, ctempty = 0, ctovf = 0;
+  if (lane < 4) S.tally[lane] = 0;
   int* const work = P.from_mid ? &P.work[5] : &P.work[0];
   const int total = P.from_mid ? P.st->mid_count : P.cell_end - P.cell_begin;
   auto original = [&](int j) { return BRUTE ? j : P.perm[j]; };
@@ -329,7 +331,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
     const float* box = SI.lo;
     const bool weighted = SI.weighted != 0;
     int mode = P.loser[si] || !finite_site(me) ? S_EMPTY : S_BUILD;
-    const unsigned amb0 = ctamb;
+    unsigned ct64 = 0, ctamb = 0, ctrefv = 0;  // this cell's, a lane's share
 
     // ---- the box: 6 planes, 8 corners (as init_cell)
     if (lane < 6) {
@@ -945,13 +947,22 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
       P.ovf_list[atomicAdd(&P.st->ovf_count, 1)] = si;
       if (P.tape) *reinterpret_cast<int4*>(P.tape + (size_t)si * kTapeStride) = make_int4(-1, 0, 0, 0);
     }
-    if (!BRUTE && __any_sync(FULL, ctamb != amb0) && lane == 0) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+    // the events of cells that this kernel finishes: those of one passed on are
+    // counted by the large-cell pass
+    if (mode <= S_EMPTY && __any_sync(FULL, (ct64 | ctrefv) != 0)) {
+      const unsigned signs = __reduce_add_sync(FULL, ct64), amb = __reduce_add_sync(FULL, ctamb),
+                     verts = __reduce_add_sync(FULL, ctrefv);
+      if (lane == 0) {
+        S.tally[0] += signs;
+        S.tally[1] += amb;
+        S.tally[2] += verts;
+        if (!BRUTE && amb) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+      }
+    }
     __syncwarp();
   }
-  ct64 = __reduce_add_sync(FULL, ct64);
-  ctamb = __reduce_add_sync(FULL, ctamb);
-  ctrefv = __reduce_add_sync(FULL, ctrefv);
   if (lane == 0) {
+    const unsigned ct64 = S.tally[0], ctamb = S.tally[1], ctrefv = S.tally[2];
     if (ct64) atomicAdd((unsigned long long*)&P.st->fp64_fallbacks, (unsigned long long)ct64);
     if (ctamb) atomicAdd((unsigned long long*)&P.st->fp64_ambiguous, (unsigned long long)ctamb);
     if (ctrefv) atomicAdd((unsigned long long*)&P.st->refined_vertices, (unsigned long long)ctrefv);
