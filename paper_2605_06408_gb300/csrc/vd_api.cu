@@ -431,7 +431,6 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   c.vol = out->volume;
   c.cen = out->centroid;
   const bool knn = (ctx->cfg.warm_start == 2 && ctx->cfg.cell_mode == 0) || uses_wide(ctx->cfg);
-  c.have_knn = knn ? 1 : 0;
   if (knn) {  // the KNN warm start's lists (App. A.6), for this build's cells
     e = launch_knn(c, ctx->knn, s);
     if (e != cudaSuccess) return VD_ERR_CUDA;

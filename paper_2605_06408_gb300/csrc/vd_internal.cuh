@@ -320,8 +320,7 @@ struct CellBuffers {
   int cell_end;          //   (all of [0, n) unless the context is partitioned)
   int* mid_list;         // [n] sorted indices of the cells left to the one-per-warp kernel
   int from_mid;          // 1: solo_kernel makes the cells of mid_list
-  int have_knn;          // the KNN lists were made in this build
-  const int* knn;        // [n * kKnn] nearest sites (sorted indices, -1 = none) for warm_start = 2
+  const int* knn;        // [n * kKnn] nearest sites (sorted indices, -1 = none)
 };
 
 constexpr int kSortHist = 8 * 256 + 64;  // digit counts and tickets at the head of the sort's scratch

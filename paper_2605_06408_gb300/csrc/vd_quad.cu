@@ -456,7 +456,7 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
           dup = dup | (act[r] & (nn == 0.f));
         }
         if (__any_sync(FULL, dup)) {
-          // duplicate positions (of another weight stratum: mark_losers sees
+          // duplicate positions (of another weight stratum: gather_sites sees
           // the others): the larger weight, then the lower index, wins
           bool lose = false;
 #pragma unroll

@@ -360,10 +360,8 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
     }
     int nv = 8, np = 6, qn = 1, cn = 0;
 
-    // ---- first sites: the KNN list if there is one (App. A.6), else the
-    // site's 32 neighbours in the sorted order (one coalesced load)
-    const bool knn = P.have_knn != 0;
-    int kid = -1, w0 = 0, w1 = 0;
+    // ---- first sites: the KNN list (App. A.6)
+    int kid = -1;
     if (BRUTE) {
       float best = INFINITY;
       for (int j = lane; j < P.n; j += 32) {
@@ -375,20 +373,15 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           kid = j;
         }
       }
-    } else if (knn) {
-      if (lane < kKnn) kid = P.knn[(size_t)si * kKnn + lane];
-    } else {
-      const int lo = SI.first, hi = SI.first + SI.count;
-      w0 = max(lo, min(si - 16, hi - 32));
-      w1 = min(hi, w0 + 32);
+    } else if (lane < kKnn) {
+      kid = P.knn[(size_t)si * kKnn + lane];
     }
     {
-      const int j = BRUTE || knn ? kid : (w0 + lane < w1 && w0 + lane != si ? w0 + lane : -1);
-      const uint32_t m = __ballot_sync(FULL, j >= 0);
-      if (j >= 0) {
+      const uint32_t m = __ballot_sync(FULL, kid >= 0);
+      if (kid >= 0) {
         const int at = __popc(m & lt);
-        S.cand[at] = P.sites[j];
-        S.cid[at] = j;
+        S.cand[at] = P.sites[kid];
+        S.cid[at] = kid;
       }
       cn = __popc(m);
     }
@@ -537,7 +530,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
             const int c = lane < 16 ? c0 : c1;
             const int ref = __shfl_sync(FULL, cref, c & 31);
             j[r] = leaf_first(ref) + (lane & 15);
-            act[r] = (c >= 0) & ((lane & 15) < leaf_count(ref)) & (j[r] != si) & ((j[r] < w0) | (j[r] >= w1));
+            act[r] = (c >= 0) & ((lane & 15) < leaf_count(ref)) & (j[r] != si);
             q[r] = P.sites[act[r] ? j[r] : si];
           }
         }
@@ -550,7 +543,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           dup = dup | (act[r] & (nn == 0.f));
         }
         if (__any_sync(FULL, dup)) {
-          // duplicate positions (of another weight stratum: mark_losers sees
+          // duplicate positions (of another weight stratum: gather_sites sees
           // the others): the larger weight, then the lower index, wins
           bool lose = false;
 #pragma unroll
@@ -601,7 +594,7 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
           break;
         }
         if (BRUTE && !first) left = left & (id != __shfl_sync(FULL, kid, id & 31));
-        if (!BRUTE && knn && !first) {
+        if (!BRUTE && !first) {
 #pragma unroll
           for (int k = 0; k < kKnn; k++) left = left & (id != __shfl_sync(FULL, kid, k));
         }
