@@ -449,10 +449,9 @@ static int run_forward(vd_ctx* ctx, const float* xyz, const float* w, int n, int
   ctx->last_stream = s;
   ctx->ev_valid = ctx->cfg.timing != 0;
   ctx->ev_backward = false;
-  const int sorts = n <= 1 ? 0 : (n <= 2048 ? 1 : (bits + 7) / 8);
   // weights, keys, sort, sites, tree (2), records, KNN, cells (1 or 2), large cells, scan, rows
-  ctx->launches = (w ? 1 : 0) + 1 + sorts + 1 + (n >= 2 ? 2 : 0) + 1 + (knn ? 1 : 0) + (quad ? 2 : 1) + 1 +
-                  (n > 8192 ? 3 : 1) + 1;
+  ctx->launches = (w ? 1 : 0) + 1 + sort_launches(n, bits) + 1 + (n >= 2 ? 2 : 0) + 1 + (knn ? 1 : 0) + (quad ? 2 : 1) +
+                  1 + scan_launches(n) + 1;
   return VD_OK;
 }
 

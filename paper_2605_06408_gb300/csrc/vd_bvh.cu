@@ -393,6 +393,8 @@ __global__ void __launch_bounds__(512) sort_small_kernel(uint64_t* __restrict__ 
   }
 }
 
+int sort_launches(int n, int bits) { return n <= 1 ? 0 : (n <= kSortSmall ? 1 : (bits + 7) / 8); }
+
 cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, int*& vals_alt, unsigned* scratch, int n,
                              int bits, DevStatus* st, cudaStream_t s) {
   if (n <= 1) return cudaSuccess;

@@ -173,6 +173,8 @@ cudaError_t launch_mesh_finish(const DevStatus* st, int64_t* nverts_out, int32_t
   return cudaGetLastError();
 }
 
+int scan_launches(int n) { return n > kScanTile ? 3 : 1; }
+
 // Exclusive scan of n counts into offsets[n+1]; the total goes to *total.
 cudaError_t launch_scan(const int* counts, int n, int32_t* offsets, long long* block_sums, long long* total,
                         DevStatus* st, cudaStream_t s) {

@@ -357,6 +357,7 @@ cudaError_t launch_pack_keys(const float* xyz, const float* w, int n, const SetI
                              int* ovf_slot, DevStatus* st, cudaStream_t s);
 size_t sort_scratch_bytes(int64_t n);
 size_t sort_clear_words(int n);
+int sort_launches(int n, int bits);
 cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, int*& vals_alt, unsigned* scratch, int n,
                              int bits, DevStatus* st, cudaStream_t s);
 cudaError_t launch_gather_sites(const float* xyz, const float* w, int* perm, int n, const SetInfo* sets, uint64_t* keys,
@@ -377,6 +378,7 @@ cudaError_t launch_csr(const CellBuffers& c, int32_t* offsets, int32_t* neighbor
 cudaError_t launch_backward(const BackBuffers& b, int num_sms, cudaStream_t s);
 cudaError_t launch_scan(const int* counts, int n, int32_t* offsets, long long* block_sums, long long* total,
                         DevStatus* st, cudaStream_t s);
+int scan_launches(int n);
 cudaError_t launch_mesh_finish(const DevStatus* st, int64_t* nverts_out, int32_t* user_status, cudaStream_t s);
 
 }  // namespace vd
