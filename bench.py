@@ -8,8 +8,8 @@ value is Mcells/s. The default workload is the largest configuration that
 fits one GPU: 20,000,000 sites in nested Gaussian shells around random
 surfaces, forward and forward+backward. Forward+backward throughput, the
 end-to-end number through the C ABI from pinned host buffers, the roofline
-of the fused kernel (and, beside it, of the large-cell pass) and the FP64 CPU
-oracle on the host cores are reported in the same JSON line.
+of the cell kernels and the FP64 CPU oracle on the host cores are reported in
+the same JSON line.
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--workload NAME]
     python bench.py --impl reference ...   # the FP64 CPU oracle, same workload
@@ -68,12 +68,23 @@ WORKLOADS = {
                   "per step, replayed from a CUDA graph",
 }
 
-# algorithmic FP32 work per counted event:
-# one vertex/plane sign test = 3 FMA; one new vertex = three cross products,
-# a determinant, three 3-term numerators and a reciprocal (51 flop); one leaf
-# candidate = its plane and support test (30 flop); one BVH child = its
-# distance, radius and bound (40 flop).
-FLOP_VTEST, FLOP_NEWV, FLOP_CAND, FLOP_NODE = 6, 51, 30, 40
+# FP32 work that a cell cannot do without: one vertex/plane sign test = 3 FMA;
+# one vertex = three cross products, a determinant, three 3-term numerators and
+# a reciprocal (51 flop); one face's plane (30 flop); one tetrahedron of the
+# volume and first moment (60 flop).
+FLOP_VTEST, FLOP_VERTEX, FLOP_PLANE, FLOP_TET = 6, 51, 30, 60
+
+
+def needed_flops(neighbour_counts) -> float:
+    """FP32 operations that the cells with these neighbour counts cannot do
+    without, whatever finds them: a cell of F faces has 2F - 4 vertices (a
+    simple polytope), each solved once and checked against each face, and a
+    tetrahedron per directed edge of a face (three a vertex). Empty cells cost
+    nothing; box faces are left out (a cell has at least 4 faces)."""
+    f = np.asarray(neighbour_counts, np.float64)
+    f = np.maximum(f[f > 0], 4.0)
+    v = 2.0 * f - 4.0
+    return float(np.sum(v * (FLOP_VERTEX + FLOP_VTEST * f + 3 * FLOP_TET) + FLOP_PLANE * f))
 
 
 def parse():
@@ -407,15 +418,13 @@ def run_ours(args):
     cap = nnz + 1024
     st = ctx.status()
 
-    # algorithmic work of one build, from a separate counting run
+    # the work of one build by its outputs, independent of the kernels that run;
+    # and the events of a counting build, whose cells another kernel makes (the
+    # timed ones count nothing)
+    flop = needed_flops(torch.diff(res.offsets).cpu().numpy())
     cctx = new_ctx(dict(cfg, counters=1))
     build(cctx, sites, weights)
     cnt = cctx.status()
-    # the main pass (fused kernel) and the large-cell pass are counted apart
-    flop = (FLOP_VTEST * cnt["vertex_tests"] + FLOP_NEWV * cnt["new_vertices"] + FLOP_CAND * cnt["candidates"]
-            + FLOP_NODE * cnt["nodes"])
-    flop_large = (FLOP_VTEST * cnt["large_vertex_tests"] + FLOP_NEWV * cnt["large_new_vertices"]
-                  + FLOP_CAND * cnt["large_candidates"] + FLOP_NODE * cnt["large_nodes"])
     del cctx
 
     def barrier():
@@ -638,8 +647,7 @@ def run_ours(args):
     fp32_peak = props.multi_processor_count * 128 * 2 * sm_max * 1e6  # FP32 lanes x FMA x clock
     cms = statistics.mean(cells_ms)
     lms = statistics.mean(large_ms) if large_ms else 0.0
-    achieved = flop / (cms * 1e-3)
-    achieved_large = flop_large / (lms * 1e-3) if lms > 0 else 0.0
+    achieved = flop / ((cms + lms) * 1e-3)
     src_hash = kernel_source_hash()
     traffic = fused_traffic_from_profiles(src_hash, args.workload)
 
@@ -689,17 +697,16 @@ def run_ours(args):
                 "transfers": "vd_copy (SM copies over NVLink-C2C) from and to pinned host buffers"},
         "gpu_launches": launches,
         "clocks": clocks,
-        "roofline": {"bound": "alu", "kernel": "quad_kernel and solo_kernel (fused traversal + cull + clip)",
+        "roofline": {"bound": "alu", "kernel": "quad_kernel, solo_kernel and big_cells_kernel (traversal + cull + clip)",
                      "achieved": achieved / 1e12, "peak": fp32_peak / 1e12, "unit": "TFLOP/s",
-                     "frac": achieved / fp32_peak, "traffic": traffic,
+                     "frac": achieved / fp32_peak, "traffic": traffic, "traffic_kernel": "quad_kernel alone",
                      "peak_source": f"{props.multi_processor_count} SMs x 128 FP32 lanes x 2 flop x {sm_max:.0f} MHz",
-                     "flop_per_launch": flop, "cells_ms": cms,
-                     "flop_source": "main-pass counters of a separate counting build (counters = 1)",
-                     "large_cell_pass": {"kernel": "big_cells_kernel", "achieved": achieved_large / 1e12,
-                                         "frac": achieved_large / fp32_peak, "flop_per_launch": flop_large,
-                                         "ms": lms}},
+                     "flop_per_step": flop, "cells_ms": cms, "large_cells_ms": lms,
+                     "flop_source": "by the step's own outputs: each cell's vertices solved once and checked against its "
+                                    "faces, the planes, the volume (no search); over both cell phases' time"},
         "phase_ms": {k: v for k, v in ctx.timings().items() if k.endswith("_ms")},
         "nnz": nnz,
+        "counters_source": "cells_kernel, in a separate build with counters = 1 (the timed kernels count no events)",
         "counters": {k: cnt[k] for k in ("candidates", "clips", "nodes", "vertex_tests", "new_vertices",
                                          "large_candidates", "large_clips", "large_nodes", "large_vertex_tests",
                                          "large_new_vertices")},
