@@ -106,10 +106,10 @@ typedef struct {
                            /*       the LBVH before the cells are built);           */
                            /*    then the traversal skips them. Default 0 (the      */
                            /*    best-first traversal reaches the nearest leaf      */
-                           /*    first); warp-per-cell form with the ablation       */
-                           /*    modes, counters or plain FP32 only: the kernels of */
+                           /*    first); warp-per-cell form only. The kernels of    */
                            /*    the default modes always start from the 8 nearest  */
-                           /*    sites                                              */
+                           /*    sites; 1 and 2 there have the large-cell pass      */
+                           /*    start from the window                              */
   int32_t cell_mode;       /* 0: one warp per cell, polytope in registers (default);*/
                            /* 1: one thread per cell, polytope in per-thread memory */
                            /*    (the paper's mapping, App. A.3: 64 vertices, 48    */
@@ -353,14 +353,18 @@ int vd_backward_mesh(vd_ctx* ctx, const float* grad_volume, const float* grad_ce
  * vd_autotune / vd_autotune_batched time candidate configurations of
  * vd_build / vd_build_batched on the caller's input and keep the fastest in
  * ctx (returned in *best when best != NULL). Coordinate descent from the
- * context's configuration over: cell_mode (warp or thread per cell),
- * verts_per_lane (polytope capacity), queue_per_lane (queue depth),
- * leaf_size, warps_per_block and warm_start; each trial is one warm-up and
- * two timed builds (CUDA events), a change is kept if >= 2% faster, at most
- * max_trials trials (<= 0: 16). cull_mode, traversal, precision, counters
- * and timing stay the caller's. The result is cached in ctx per (floor(log2 n), any
- * set weighted, set-count class); a later call with the same key returns
- * the cached configuration without trials unless flags has VD_TUNE_FORCE.
+ * context's configuration over those knobs that its kernels read: cell_mode
+ * (warp or thread per cell); in the default modes warps_per_block (2 or 4)
+ * and, if the build has cells for the large-cell pass, warm_start (on or off)
+ * and leaf_size; with an ablation mode, counters or plain FP32 warm_start,
+ * verts_per_lane (polytope capacity), queue_per_lane (queue depth), leaf_size
+ * and warps_per_block; in the thread form leaf_size. The other knobs stay as
+ * they are. Each trial is one warm-up and two timed builds (CUDA events), a
+ * change is kept if >= 2% faster, at most max_trials trials (<= 0: 16).
+ * cull_mode, traversal, precision, counters and timing stay the caller's. The
+ * result is cached in ctx per (floor(log2 n), any set weighted, set-count
+ * class, those four modes); a later call with the same key returns the cached
+ * configuration without trials unless flags has VD_TUNE_FORCE.
  *
  * Synchronises the host (it reads timings); not capturable into a CUDA
  * graph: tune first, then capture vd_build / vd_build_batched. Allocates and

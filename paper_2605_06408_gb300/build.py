@@ -44,7 +44,7 @@ def build(force: bool = False, extra: list[str] | None = None, verbose: bool = F
     """Compile and link libvd.so; returns its path."""
     os.makedirs(OUT, exist_ok=True)
     srcs = [os.path.join(CSRC, s) for s in SOURCES]
-    hdrs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith(".cuh")]
+    hdrs = [os.path.join(CSRC, f) for f in os.listdir(CSRC) if f.endswith((".cuh", ".h"))]
     hdrs.append(os.path.join(ROOT, "include", "vd.h"))
     if not force and os.path.exists(LIB):
         t = os.path.getmtime(LIB)

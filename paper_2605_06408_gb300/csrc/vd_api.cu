@@ -13,6 +13,7 @@
 #include <tuple>
 
 #include "vd_big.cuh"
+#include "vd_tune.h"
 
 using namespace vd;
 
@@ -112,8 +113,8 @@ struct vd_ctx {
   // large-cell tape: polytopes of the cells past the register path
   char* btape = nullptr;
   int64_t btape_cap = 0;
-  // autotuner: best configuration per (log2 n, weighted, set count)
-  std::map<std::tuple<int, int, int>, vd_config> tuned;
+  // autotuner: best configuration per (log2 n, weighted, set count, kernels)
+  std::map<std::tuple<int, int, int, int>, vd_config> tuned;
   // partition of the cells (vd_set_partition): this context builds part
   // `part` of `nparts` contiguous ranges of the Morton-sorted order
   int part = 0;
@@ -796,26 +797,25 @@ int vd_ambiguous_cells(vd_ctx* ctx, int64_t* cells, int64_t capacity, int64_t* c
 //
 // Coordinate descent over the kernel form and its capacities: starting from
 // the context's configuration, each knob in turn (cell form, warm start,
-// polytope capacity, queue depth, leaf size, block size) takes each of
-// its other values; a trial is one warm-up build then the faster of two
+// polytope capacity, queue depth, leaf size, block size) takes each of its
+// other values that the kernels of the configuration so far read
+// (vd_tune.h); a trial is one warm-up build then the faster of two
 // timed builds (CUDA events on the caller's stream) of the caller's input,
 // and a value is kept if it is at least 2% faster. A configuration under
-// which a cell fails (error other than neighbour capacity) is skipped.
+// which a cell fails (error other than neighbour capacity) is skipped. The
+// kernels timed are those that the caller's builds run: its ablation modes,
+// counters and precision stay on, and the cached result holds for them only.
 static int autotune(vd_ctx* ctx, int64_t n, int nsets, int weighted, const std::function<int(const vd_out*)>& build,
                     int32_t max_trials, int32_t flags, vd_config* best, cudaStream_t s) {
   const vd_config user = ctx->cfg;
   int lg = 0;
   while ((int64_t(1) << (lg + 1)) <= n) lg++;
-  const auto key = std::make_tuple(lg, weighted, nsets > 1 ? 1 + (nsets > 64) : 0);
+  const auto key = std::make_tuple(lg, weighted, nsets > 1 ? 1 + (nsets > 64) : 0, tune_form(user));
   if (!(flags & VD_TUNE_FORCE)) {
     auto it = ctx->tuned.find(key);
     if (it != ctx->tuned.end()) {
       vd_config c = it->second;
-      c.counters = user.counters;
       c.timing = user.timing;
-      c.cull_mode = user.cull_mode;
-      c.traversal = user.traversal;
-      c.precision = user.precision;
       c.tape = user.tape;
       ctx->cfg = c;
       if (best) *best = c;
@@ -841,8 +841,8 @@ static int autotune(vd_ctx* ctx, int64_t n, int nsets, int weighted, const std::
   cudaEventCreate(&e0);
   cudaEventCreate(&e1);
   int trials = 0;
+  bool trial_large = false;  // the last trial had cells for the large-cell pass
   auto trial = [&](vd_config c, float& ms) -> bool {
-    c.counters = 0;
     c.timing = 0;
     if (check_config(&c) != VD_OK) return false;
     ctx->cfg = c;
@@ -851,6 +851,7 @@ static int autotune(vd_ctx* ctx, int64_t n, int nsets, int weighted, const std::
     vd_status st;
     if (vd_get_status(ctx, &st) != VD_OK) return false;
     if (st.error != VD_OK && st.error != VD_ERR_CAPACITY) return false;
+    trial_large = st.overflow_cells > 0;
     ms = INFINITY;
     for (int r = 0; r < 2; r++) {
       cudaEventRecord(e0, s);
@@ -872,32 +873,21 @@ static int autotune(vd_ctx* ctx, int64_t n, int nsets, int weighted, const std::
     cur.cull_mode = user.cull_mode;
     cur.traversal = user.traversal;
     cur.precision = user.precision;
+    cur.counters = user.counters;
     if (!trial(cur, cur_ms)) rc = VD_ERR_CELL_OVERFLOW;
   }
   if (rc == VD_OK) {
-    struct Knob {
-      int32_t vd_config::*field;
-      int values[3];
-      int count;
-      bool warp_only;
-    };
-    // the warm start comes before the leaf size: the best leaf size depends
-    // on it (with the KNN start, larger leaves win on every workload here)
-    const Knob knobs[] = {
-        {&vd_config::cell_mode, {0, 1, 0}, 2, false},     {&vd_config::warm_start, {0, 1, 2}, 3, true},
-        {&vd_config::verts_per_lane, {2, 4, 0}, 2, true}, {&vd_config::queue_per_lane, {2, 4, 8}, 3, true},
-        {&vd_config::leaf_size, {8, 16, 32}, 3, false},   {&vd_config::warps_per_block, {2, 4, 8}, 3, true},
-    };
-    for (const Knob& k : knobs) {
-      if (k.warp_only && cur.cell_mode != 0) continue;
-      for (int v = 0; v < k.count && trials < max_trials; v++) {
-        if (cur.*(k.field) == k.values[v]) continue;
+    bool large = trial_large;
+    for (int k = 0; k < kTuneKnobs; k++) {
+      for (const TuneValue& v : tune_values(cur, k, large)) {
+        if (trials >= max_trials) break;
         vd_config c = cur;
-        c.*(k.field) = k.values[v];
+        c.*(v.field) = v.value;
         float ms = INFINITY;
         if (trial(c, ms) && ms < 0.98f * cur_ms) {
           cur = c;
           cur_ms = ms;
+          large = trial_large;
         }
       }
     }
@@ -908,7 +898,6 @@ static int autotune(vd_ctx* ctx, int64_t n, int nsets, int weighted, const std::
   cudaFree(mem);
   // the trial builds' outputs are gone: no forward state for vd_backward
   ctx->have_forward = false;
-  cur.counters = user.counters;
   cur.timing = user.timing;
   if (rc != VD_OK) {
     ctx->cfg = user;

@@ -24,6 +24,7 @@
 #include <functional>
 
 #include "vd_big.cuh"
+#include "vd_tune.h"
 
 namespace vd {
 
@@ -1061,12 +1062,6 @@ __global__ void __launch_bounds__(32 * kBigWarpsPerBlock, kBigBlocksPerSm) big_c
     if (GEN && P.cfg.counters) ct.vtests += tested;
   }
   flush_counters(P, ct, lane, empties, 0, failed);
-}
-
-// A configuration that reads the ablation modes, the event counters or plain
-// FP32 runs the generic instantiations.
-static bool generic_config(const vd_config& g) {
-  return g.cull_mode != 0 || g.traversal != 0 || g.counters != 0 || g.precision != 0;
 }
 
 // The kernels that walk the 8-wide tree (vd_quad.cu, vd_solo.cu) fold the
