@@ -333,6 +333,17 @@ def kernel_source_hash() -> str:
     return hsh.hexdigest()[:16]
 
 
+def plain_fp32_config(tuned: dict, overrides: str) -> dict:
+    """The configuration of the plain-FP32 build: the tuned one describes the
+    kernels of the default modes, which read neither the leaf size nor the warm
+    start of the traversal; the kernel of plain FP32 does. Leaves of 32 and the
+    KNN start (surfaces2M: 505 ms against 927 with the defaults; tuning a build
+    of 20 million sites in plain FP32 takes minutes), unless the caller says
+    otherwise."""
+    own = json.loads(overrides) if overrides else {}
+    return {**tuned, "leaf_size": 32, "warm_start": 2, **own, "timing": 0, "precision": 1}
+
+
 def accuracy_sample(sess, n: int, sample: int, seed: int = 11):
     """(cells, oracle result) for `sample` seeded cells of a set of n sites."""
     from paper_2605_06408_gb300 import workloads as W
@@ -529,7 +540,7 @@ def run_ours(args):
                 ts.append(e0.elapsed_time(e1))
             return statistics.mean(ts), out
 
-        f32 = vd.Context(local, dict(cfg, timing=0, precision=1))
+        f32 = vd.Context(local, plain_fp32_config(cfg, args.config))
         # plain FP32 derails on ill-conditioned cells and can be much slower:
         # one timed build after the warm-up on large inputs
         f32_ms, r32 = timed(lambda: build(f32, sites, weights, cap * 2, sync=False), reps=3 if n <= 2_000_000 else 1)

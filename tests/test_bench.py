@@ -29,3 +29,13 @@ def test_achieved_rate_reads_no_event_counter():
     src = inspect.getsource(bench.run_ours)
     used = [line for line in src.splitlines() if "flop" in line or "achieved" in line]
     assert used and not any("cnt[" in line for line in used)
+
+
+def test_plain_fp32_form_has_its_own_knobs():
+    """Those that the tuner leaves alone in the default modes are read by the
+    kernel of plain FP32."""
+    tuned = {"leaf_size": 16, "warm_start": 0, "warps_per_block": 2, "precision": 0, "timing": 1}
+    cfg = bench.plain_fp32_config(tuned, "")
+    assert cfg == {"leaf_size": 32, "warm_start": 2, "warps_per_block": 2, "precision": 1, "timing": 0}
+    assert bench.plain_fp32_config(tuned, '{"leaf_size": 8}')["leaf_size"] == 8
+    assert "plain_fp32_config(cfg" in inspect.getsource(bench.run_ours)
