@@ -13,8 +13,8 @@
 // 380 us; the cells that outgrow 48 vertices of 1M sites in clusters and the
 // large-cell pass after it, 7.7 ms of that pass before -> 3.0 ms.
 // Polytope, planes, queue and candidates are in shared memory (11 KB a warp);
-// up to 192 vertices and 128 planes. Larger cells, and cells whose walk
-// outgrows the queue, go to the large-cell pass.
+// up to 192 vertices and 128 planes. Larger cells, and cells whose walk is long
+// or outgrows the queue, go to the large-cell pass.
 #include "vd_walk.cuh"
 
 namespace vd {
@@ -28,6 +28,15 @@ constexpr int kSC = 96;   // candidates
 constexpr int kST = 23;   // candidates at which the walk stops to clip (a step adds up to 64)
 constexpr int kSF = 39;   // faces of a cell whose edges are looked up in a table at the end
 constexpr int kSCone = 40;  // node visits (of up to four nodes) after which the cone test is made
+// Node visits after which a cell goes to the large-cell pass. They take 4.6 us
+// each, one warp at work on them long after the others (a cell at the hull of a
+// tight cluster that sees the whole empty box); there up to eight warps share a
+// cell's filters, and such sets have heavier cells in that pass anyway. Builds
+// without a limit, with 2,000 and with 1,000: 300,000 sites in 0.1% of each side
+// 194, 179 and 175 ms, in a ball of 5% 107.8, 109.1 and 106.6, one cluster of
+// sigma 0.01 86.4, 78.8 and 77.4, five clusters 52.0, 48.9 and 46.2; but 20,000 on
+// a shell 8.7, 8.7 and 18.3 (its only cell past 1,000 took 9.7 ms in that pass).
+constexpr int kSWalk = 2000;
 static_assert(kST + 1 + 64 <= kSC, "room for a step's leaves");
 
 struct __align__(16) SoloCell {
@@ -463,7 +472,10 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
               finished = true;
               break;
             }
-            steps++;
+            if (++steps > kSWalk) {
+              mode = S_FAR;
+              break;
+            }
             uint32_t todo = 255u;
             int ref = lane < 8 ? cur : -1;
             if (cur < 0) ref = solo_pop(S, qn, todo);
