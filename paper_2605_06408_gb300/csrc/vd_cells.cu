@@ -1070,9 +1070,17 @@ bool uses_wide(const vd_config& g) { return g.cell_mode == 0 && !generic_config(
 
 // Four cells per warp from 192 sites per SM on (29,184 on GB300): a build of
 // fewer is bound by the latency of one warp's work, which is one cell here and
-// four there. Cells of uniform sites, one per warp and four: 10,000 sites 0.38
-// and 0.55 ms, 29,000 1.00 and 0.81 ms, 300,000 8.8 and 5.5 ms. By the sites of
-// the whole diagram, so that the parts of a partition agree with it to the last bit.
+// four there. Where the two lines cross hangs on the sites. All cells of a build,
+// one per warp and four, in ms:
+//   sites                      12,000       18,000       24,000       29,000       36,000
+//   uniform                 0.45, 0.48   0.67, 0.63   0.83, 0.71   0.96, 0.78   1.21, 0.96
+//   uniform, Gauss weights  0.51, 0.61   0.73, 0.69   0.96, 0.87   1.11, 0.91   1.40, 1.04
+//   64 uneven clusters      1.12, 1.59   1.36, 1.97   1.78, 1.99   2.14, 2.25   2.37, 2.45
+//   5 tight clusters        1.26, 3.63   1.73, 3.91   2.17, 4.20   2.26, 4.35   2.81, 4.64
+// and 300,000 uniform sites 8.8, 5.5. Even sites gain from four at 16,000 already,
+// clusters (a few long walks, which all four cells of a warp wait for) only well
+// past 36,000; the line stands between. By the sites of the whole diagram, so that
+// the parts of a partition agree with it to the last bit.
 bool uses_quad(const vd_config& g, int n, int num_sms) { return uses_wide(g) && n >= 192 * num_sms; }
 
 template <int VPL, int PCAP, int QPL>

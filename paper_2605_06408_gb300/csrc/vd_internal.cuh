@@ -21,8 +21,14 @@ constexpr unsigned FULL = 0xffffffffu;
 constexpr int kMaxLeaf = 32;            // leaf sizes 1..32 (one site per lane)
 constexpr int kMaxSites = 1 << 26;      // leaf refs pack the first site in 26 bits
 constexpr int kMaxSets = 1024;
-constexpr int kBigWarpsPerBlock = 8;  // large-cell path: blocks of this many warps,
-constexpr int kBigBlocksPerSm = 1;     // this many per SM (one arena per warp)
+// Large-cell path: blocks of this many warps, this many per SM (one arena of 2.1
+// MB per warp). Two blocks (at 128 registers instead of 160) help a pass over
+// thousands of mid-sized cells, which only the ablation modes still have (2M
+// sites on surfaces, counters 18.8 -> 16.6 ms of 123, depth-first 39.0 -> 36.8 of
+// 159), and slow it where few heavy cells or plain FP32 bound it (269 -> 277 of
+// 505; 200,000 heavy-tailed weights 135 -> 138 of 156 under isotropic culling).
+constexpr int kBigWarpsPerBlock = 8;
+constexpr int kBigBlocksPerSm = 1;
 constexpr uint32_t kEmptyTri = 0xffffffffu;
 #ifndef VD_KNN
 #define VD_KNN 8
