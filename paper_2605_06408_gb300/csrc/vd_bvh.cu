@@ -432,7 +432,8 @@ cudaError_t radix_sort_pairs(uint64_t*& keys, uint64_t*& keys_alt, int*& vals, i
 // arrays: every place takes the input's own order instead, with keys of the
 // set alone (sorted, so the tree over them is a valid one), and every site is a
 // loser, so that no cell is made of it: the build ends with empty rows and
-// VD_ERR_TIMEOUT. One place, for the host too (that order is tested there).
+// VD_ERR_TIMEOUT. (This function makes place k. It is compiled for the host too,
+// where a test runs it on such arrays.)
 __host__ __device__ inline void gather_site(const float* xyz, const float* w, int* perm, int n, const SetInfo* sets,
                                             uint64_t* keys, int set_shift, int nsets, bool failed, float4* sites,
                                             int* inv, unsigned char* loser, int k) {
