@@ -776,7 +776,7 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
     if (!own) mode = M_IDLE;
     if (mode == M_EMPTY) {
       if (gl == 0) {
-        S.tally[T_EMPTY]++;
+        atomicAdd(&S.tally[T_EMPTY], 1u);
         P.counts[orig] = 0;
         P.vol[orig] = 0.0f;
         P.cen[3 * (size_t)orig] = me.x;
@@ -916,7 +916,7 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
             oy += Y6 * iv;
             oz += Z6 * iv;
           }
-          if (gl == 0) S.tally[T_VOLS]++;
+          if (gl == 0) atomicAdd(&S.tally[T_VOLS], 1u);
         }
       }
       if (!need64 && V > 0.0f) {
@@ -935,15 +935,12 @@ __global__ void __launch_bounds__(128, 4) quad_kernel(CellBuffers P) {
     // the events of cells that this kernel finishes: of one passed on, the next
     // kernel counts them, of a neighbouring part's cell, that part's build
     const bool kept = mode == M_BUILD || mode == M_EMPTY;
-    if (__any_sync(FULL, kept && (ct64 | ctrefv) != 0)) {
-      const unsigned signs = (unsigned)group_add((int)ct64), amb = (unsigned)group_add((int)ctamb),
-                     verts = (unsigned)group_add((int)ctrefv);
-      if (kept && gl == 0) {
-        S.tally[T_SIGNS] += signs;
-        S.tally[T_AMB] += amb;
-        S.tally[T_VERTS] += verts;
-        if (amb) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
-      }
+    const uint32_t am = group_ballot(kept && ctamb != 0);
+    if (am && gl == 0) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+    if (kept && ctrefv) atomicAdd(&S.tally[T_VERTS], ctrefv);
+    if (kept && ct64) {
+      atomicAdd(&S.tally[T_SIGNS], ct64);
+      atomicAdd(&S.tally[T_AMB], ctamb);
     }
     __syncwarp();
   }

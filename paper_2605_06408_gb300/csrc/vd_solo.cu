@@ -954,14 +954,12 @@ __global__ void __launch_bounds__(128, 4) solo_kernel(CellBuffers P) {
     }
     // the events of cells that this kernel finishes: those of one passed on are
     // counted by the large-cell pass
-    if (mode <= S_EMPTY && __any_sync(FULL, (ct64 | ctrefv) != 0)) {
-      const unsigned signs = __reduce_add_sync(FULL, ct64), amb = __reduce_add_sync(FULL, ctamb),
-                     verts = __reduce_add_sync(FULL, ctrefv);
-      if (lane == 0) {
-        S.tally[0] += signs;
-        S.tally[1] += amb;
-        S.tally[2] += verts;
-        if (!BRUTE && amb) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+    if (mode <= S_EMPTY) {
+      if (!BRUTE && __any_sync(FULL, ctamb != 0) && lane == 0) record_ambiguous(P.st, P.amb_list, P.amb_cap, orig);
+      if (ctrefv) atomicAdd(&S.tally[2], ctrefv);
+      if (ct64) {
+        atomicAdd(&S.tally[0], ct64);
+        atomicAdd(&S.tally[1], ctamb);
       }
     }
     __syncwarp();
