@@ -157,8 +157,10 @@ typedef struct {
   int64_t new_vertices;       /* counters=1: vertices created                       */
   int64_t refined_vertices;   /* ill-conditioned vertices recomputed in FP64         */
   int64_t refined_volumes;    /* cells whose volume/centroid were integrated in FP64 */
-  int64_t overflow_reason[4]; /* register-path overflows by cause: queue, vertices,  */
-                              /*   planes, neighbours (> 64 per row)                */
+  int64_t overflow_reason[4]; /* cells for the large-cell pass by cause: queue (or,  */
+                              /*   in the default modes, a walk of over 2,000 node  */
+                              /*   visits), vertices, planes, neighbours (no room   */
+                              /*   for a long row)                                  */
   int64_t large_candidates;   /* counters=1: the same five counts for the           */
   int64_t large_clips;        /*   large-cell pass (cells that left the register    */
   int64_t large_nodes;        /*   path), including the vertex tests its helping    */
