@@ -159,8 +159,8 @@ typedef struct {
   int64_t refined_volumes;    /* cells whose volume/centroid were integrated in FP64 */
   int64_t overflow_reason[4]; /* cells for the large-cell pass by cause: queue (or,  */
                               /*   in the default modes, a walk of over 2,000 node  */
-                              /*   visits), vertices, planes, neighbours (no room   */
-                              /*   for a long row)                                  */
+                              /*   visits), vertices, planes, neighbours (> 64 per   */
+                              /*   row; in the default modes: no room for such one) */
   int64_t large_candidates;   /* counters=1: the same five counts for the           */
   int64_t large_clips;        /*   large-cell pass (cells that left the register    */
   int64_t large_nodes;        /*   path), including the vertex tests its helping    */
